@@ -212,6 +212,34 @@ int adha_section_backward(const adha_schema* schema, int64_t n, const adha_layou
                           void* const* state_ptrs, void* const* grad_ptrs, const adha_section* section,
                           const void* save, adha_stream stream);
 
+/*
+ * A run of AXPB, MUL and TANH sections and its gradient, in one pass over the
+ * records each (paper Section 2, the combine edge): the same bytes as
+ * adha_run_section with `save` for each section and adha_section_backward for
+ * each in reverse, without a saved value per section.  All fields must be fp32.
+ *
+ * adha_chain_plan: how many of sections[0..n_sec) one run takes from the first on
+ * (*n_run, at least 1: up to 128, fewer where the reverse walk would have to
+ * keep too many values) and the bytes of the run's saved buffer for n records
+ * (*saved_bytes).  Host only.
+ *
+ * adha_chain_forward: runs sections[0..n_sec) (at most adha_chain_plan's n_run) in
+ * place and writes into `saved` (device, 16-byte aligned) the values that the
+ * fields written by the run had before it.  Async.
+ *
+ * adha_chain_backward: puts the state back to what it was before the run (from
+ * `saved`) and carries the adjoints grad_in (device, as grad_ptrs of
+ * adha_section_backward) through the run in reverse into grad_out: the same
+ * buffers as grad_in (in place), or others, which must not overlap them.  Async.
+ */
+int adha_chain_plan(const adha_schema* schema, int64_t n, const adha_section* sections, int32_t n_sec, int32_t* n_run,
+                    size_t* saved_bytes);
+int adha_chain_forward(const adha_schema* schema, int64_t n, const adha_layout* layout, void* const* ptrs,
+                       const adha_section* sections, int32_t n_sec, float* saved, adha_stream stream);
+int adha_chain_backward(const adha_schema* schema, int64_t n, const adha_layout* layout, void* const* state_ptrs,
+                        const void* const* grad_in, void* const* grad_out, const adha_section* sections, int32_t n_sec,
+                        const float* saved, adha_stream stream);
+
 /* ----------------------------------------------------------- planning (host) */
 
 /* Options of candidate generation (ODS) and layout choice (PDL). */
@@ -744,8 +772,8 @@ int adha_gather_probe(const void* table, const int32_t* perm, void* out, int64_t
 
 /* One kernel launch seen by the profiler.  kind: 0 remap, 1 section, 2 section
  * backward, 3 batched remap, 4 fused run, 5 gather probe, 6 section run as a
- * one-section run specialised at run time; op: the section's
- * adha_op (0 for remaps; the number of sections for a fused run; the element
+ * one-section run specialised at run time, 7 chain run, 8 chain run backward; op: the section's
+ * adha_op (0 for remaps; the number of sections for a fused or chain run; the element
  * bytes for the probe); bytes:
  * the algorithmic bytes the launch had to move (data bytes of the moved or
  * accessed fields, not padding or untouched fields); ms: its duration between

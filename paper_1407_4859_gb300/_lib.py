@@ -93,6 +93,12 @@ SIGNATURES = {
                                                ctypes.POINTER(adha_section), _I32, _P]),
     "adha_section_backward": (ctypes.c_int, [ctypes.POINTER(adha_schema), _I64, ctypes.POINTER(adha_layout), _PP,
                                              _PP, ctypes.POINTER(adha_section), _P, _P]),
+    "adha_chain_plan": (ctypes.c_int, [ctypes.POINTER(adha_schema), _I64, ctypes.POINTER(adha_section), _I32,
+                                       ctypes.POINTER(_I32), ctypes.POINTER(ctypes.c_size_t)]),
+    "adha_chain_forward": (ctypes.c_int, [ctypes.POINTER(adha_schema), _I64, ctypes.POINTER(adha_layout), _PP,
+                                          ctypes.POINTER(adha_section), _I32, _P, _P]),
+    "adha_chain_backward": (ctypes.c_int, [ctypes.POINTER(adha_schema), _I64, ctypes.POINTER(adha_layout), _PP, _PP,
+                                           _PP, ctypes.POINTER(adha_section), _I32, _P, _P]),
     "adha_tune_override": (ctypes.c_int, [_I32]),
     "adha_batched_create": (ctypes.c_int, [_I32, ctypes.POINTER(adha_remap_desc), _I32, _P, ctypes.POINTER(_P)]),
     "adha_batched_workspace_bytes": (ctypes.c_size_t, [_P]),

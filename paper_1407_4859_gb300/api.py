@@ -135,6 +135,26 @@ def adha_section_backward(schema, n, layout, state_bufs, grad_bufs, section, sav
                                             save.data_ptr(), _stream_ptr(stream)), "adha_section_backward")
 
 
+def adha_chain_plan(schema, n, sections):
+    """(sections that one chain run takes from the first on, bytes of its saved buffer); sections: an
+    adha_section array."""
+    m, need = ctypes.c_int32(0), ctypes.c_size_t(0)
+    check(_lib.load().adha_chain_plan(ctypes.byref(schema.c), int(n), sections, len(sections), ctypes.byref(m),
+                                      ctypes.byref(need)), "adha_chain_plan")
+    return m.value, need.value
+
+
+def adha_chain_forward(schema, n, layout, bufs, sections, saved, stream=None):
+    check(_lib.load().adha_chain_forward(ctypes.byref(schema.c), int(n), ctypes.byref(layout.c), _ptrs(bufs), sections,
+                                         len(sections), saved.data_ptr(), _stream_ptr(stream)), "adha_chain_forward")
+
+
+def adha_chain_backward(schema, n, layout, state_bufs, grad_in, grad_out, sections, saved, stream=None):
+    check(_lib.load().adha_chain_backward(ctypes.byref(schema.c), int(n), ctypes.byref(layout.c), _ptrs(state_bufs),
+                                          _ptrs(grad_in), _ptrs(grad_out), sections, len(sections), saved.data_ptr(),
+                                          _stream_ptr(stream)), "adha_chain_backward")
+
+
 def adha_tune_override(chunk_records=0):
     check(_lib.load().adha_tune_override(int(chunk_records)), "adha_tune_override")
 
@@ -543,7 +563,7 @@ def _view_device(ptr, nbytes):
 
 
 KINDS = {0: "remap", 1: "section", 2: "section_backward", 3: "batched_remap", 4: "fused", 5: "gather_probe",
-         6: "section_specialised"}
+         6: "section_specialised", 7: "chain", 8: "chain_backward"}
 
 
 def adha_gather_probe(table, perm, out, rec_bytes=16, stream=None):
@@ -564,7 +584,7 @@ def adha_profile_stop(max_records=4096):
     n = ctypes.c_int32(0)
     check(_lib.load().adha_profile_stop(recs, max_records, ctypes.byref(n)), "adha_profile_stop")
     return [dict(kind=KINDS.get(recs[k].kind, recs[k].kind),
-                 op=recs[k].op if recs[k].kind in (4, 5) else OP_NAMES.get(recs[k].op, recs[k].op),
+                 op=recs[k].op if recs[k].kind in (4, 5, 7, 8) else OP_NAMES.get(recs[k].op, recs[k].op),
                  bytes=recs[k].bytes, ms=recs[k].ms) for k in range(min(n.value, max_records))]
 
 

@@ -7,20 +7,23 @@ fp32, so a group's struct is k contiguous floats).  Three autograd Functions:
   backward is the inverse remap of the incoming gradients (the same byte permutation, reversed).
   Groups the two layouts share are not inputs or outputs of the Function: the same tensor carries
   the data and its gradient straight through.
-* SegmentFn: runs a run of axpb / mul / tanh sections in place in one layout, saving each value a
-  section overwrites; its backward walks the sections in reverse with the adjoint kernel
-  (adha_section_backward), which restores the overwritten field and propagates the adjoints.
+* SegmentFn: runs a run of axpb / mul / tanh sections in place in one layout, as chain runs
+  (adha_chain_forward) that save what the written fields held before the run; its backward
+  (adha_chain_backward) puts that back, runs the sections again on chip and walks them in reverse,
+  propagating the adjoints.
 * CopyFn: a copy of the state by the remap kernel, where the first section keeps the input layout.
 
 DifferentiableProgram strings them together for a whole program under a layout plan.  Every
 forward and backward step runs in the library's kernels; PyTorch only allocates and orders them.
-Memory: the forward keeps one saved field (n floats) per section and every layout's moved groups;
+Memory: the forward keeps one saved field (n floats) per written field of each run and every layout's
+moved groups;
 the backward hands the program's state back to what it was before each segment, in place, so the
 forward outputs hold the input-side values once backward() has run (copy them first if needed).
 """
 import torch
 
-from .api import c_section, adha_remap, adha_run_section, adha_section_backward
+from ._lib import adha_section
+from .api import adha_chain_backward, adha_chain_forward, adha_chain_plan, adha_remap, adha_run_section, c_section
 
 
 def _copy(schema, n, layout, groups):
@@ -104,33 +107,46 @@ class SegmentFn(torch.autograd.Function):
     @staticmethod
     def forward(ctx, meta, *groups):
         schema, n, layout, sections = meta
-        saves = []
-        for s in sections:
-            cs = c_section(s)
-            save = torch.empty(n, dtype=torch.float32, device="cuda")
-            adha_run_section(schema, n, layout, list(groups), cs, save=save)
-            saves.append((cs, save))
+        runs = []
+        k = 0
+        if any(schema.dtypes):   # other types than fp32 (forward only): chain runs do not take them
+            for s in sections:
+                save = torch.empty(n, dtype=torch.float32, device="cuda")
+                adha_run_section(schema, n, layout, groups, c_section(s), save=save)
+                runs.append(((adha_section * 1)(c_section(s)), save))
+            k = len(sections)
+        while k < len(sections):
+            secs = (adha_section * (len(sections) - k))(*[c_section(s) for s in sections[k:]])
+            m, need = adha_chain_plan(schema, n, secs)
+            if m < len(secs):
+                secs = (adha_section * m)(*secs[:m])
+            saved = torch.empty(need // 4, dtype=torch.float32, device="cuda")
+            adha_chain_forward(schema, n, layout, groups, secs, saved)
+            runs.append((secs, saved))
+            k += m
         ctx.meta = (schema, n, layout)
-        ctx.state = groups          # updated in place; the backward restores it section by section
-        ctx.saves = saves
+        ctx.state = groups          # updated in place; the backward restores it run by run
+        ctx.runs = runs
         ctx.mark_dirty(*groups)
         return groups
 
     @staticmethod
     def backward(ctx, *grads):
         schema, n, layout = ctx.meta
-        # the adjoint kernels update the gradients in place: work on copies of the incoming ones
         g = [x.contiguous() if x is not None else torch.zeros((n, len(layout.groups[k])), dtype=torch.float32,
                                                               device="cuda")
              for k, x in enumerate(grads)]
-        g = _copy(schema, n, layout, g)
-        for cs, save in reversed(ctx.saves):
-            adha_section_backward(schema, n, layout, list(ctx.state), g, cs, save)
+        # the incoming gradients stay as they are: the last run's pass writes buffers of its own,
+        # which the earlier runs then update in place
+        out = [torch.empty_like(x) for x in g]
+        for secs, saved in reversed(ctx.runs):
+            adha_chain_backward(schema, n, layout, ctx.state, g, out, secs, saved)
+            g = out
         # the state tensors' grad_fn refers to ctx: drop them here, or the step's memory waits for
         # Python's cycle collector
-        ctx.saves = None
+        ctx.runs = None
         ctx.state = None
-        return (None,) + tuple(g)
+        return (None,) + tuple(out)
 
 
 class DifferentiableProgram:

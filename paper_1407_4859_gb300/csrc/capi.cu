@@ -391,9 +391,11 @@ static int cached_occupancy(int kind, size_t smem, int* blocks) {
       return 0;
     }
   }
-  // kinds: < 100 remap (direct or not), 100 + op section, 200 + 10*M + vec + 2*km fused run
+  // kinds: < 100 remap (direct or not), 100 + op section, 200 + 10*M + vec + 2*km fused run,
+  // 300 + 10*M + backward chain run
   const int rc = kind < 100    ? remap_occupancy(kind, smem, blocks)
                  : kind < 200 ? section_occupancy(kind - 100, smem, blocks)
+                 : kind >= 300 ? chain_occupancy((kind - 300) / 10, (kind - 300) % 10 != 0, smem, blocks)
                               : fused_occupancy((kind - 200) / 10, ((kind - 200) % 10) & 1, ((kind - 200) % 10) >> 1,
                                                 smem, blocks);
   if (rc) return rc;
@@ -1077,6 +1079,179 @@ int fused_jit_args(const Layout& L, const adha_section* s, int m, int64_t n, int
   return rc;
 }
 
+// ------------------------------------------------------------------ chain runs
+// Whether sections s[0..m) may be one chain run: fp32 fields only, axpb / mul / tanh sections.
+static int check_chain(const Layout& L, const adha_section* s, int m, int64_t n) {
+  if (!s) return fail(ADHA_EINVAL, "sections are NULL");
+  if (m < 1) return fail(ADHA_EINVAL, "a chain run holds at least one section (got %d)", m);
+  for (int f = 0; f < L.F; ++f)
+    if (L.dtype[f] != ADHA_F32) return fail(ADHA_EINVAL, "a chain run needs fp32 fields (field %d is not)", f);
+  for (int k = 0; k < m; ++k) {
+    if (s[k].op != ADHA_OP_AXPB && s[k].op != ADHA_OP_MUL && s[k].op != ADHA_OP_TANH)
+      return fail(ADHA_EINVAL, "chain section %d is not an axpb, mul or tanh section", k);
+    if (int rc = check_section(L, &s[k], n, true)) return rc;
+  }
+  return 0;
+}
+
+// Operands of a chain section: x, y (x where the op has one operand), z.
+static void chain_operands(const adha_section* s, int* x, int* y, int* z) {
+  *x = s->arg[0];
+  *y = s->op == ADHA_OP_MUL ? s->arg[1] : s->arg[0];
+  *z = s->op == ADHA_OP_MUL ? s->arg[2] : s->arg[1];
+}
+
+// What the reverse walk needs of each field's versions (version f < F: the field's value before the
+// run; F + k: what section k writes).  adj: read by a mul (its adjoint multiplies by the operands)
+// or made by a tanh (its adjoint takes the result).  live: adj, or an operand on the way to one.
+// The backward pass runs only the live sections again; each puts the value it overwrites on the
+// tape if that value is adj.  tape[k] = slot or -1.  Returns the number of slots.
+static int chain_tape(int F, const adha_section* s, int m, std::vector<int>* tape, std::vector<bool>* live_sec) {
+  std::vector<int> cur(F), vx(m), vy(m);
+  std::vector<bool> adj(F + m, false);
+  for (int f = 0; f < F; ++f) cur[f] = f;
+  for (int k = 0; k < m; ++k) {
+    int x, y, z;
+    chain_operands(&s[k], &x, &y, &z);
+    vx[k] = cur[x];
+    vy[k] = cur[y];
+    if (s[k].op == ADHA_OP_MUL) adj[vx[k]] = adj[vy[k]] = true;
+    if (s[k].op == ADHA_OP_TANH) adj[F + k] = true;
+    cur[z] = F + k;
+  }
+  std::vector<bool> live = adj;
+  for (int k = m - 1; k >= 0; --k)
+    if (live[F + k]) live[vx[k]] = live[vy[k]] = true;
+  for (int f = 0; f < F; ++f) cur[f] = f;
+  tape->assign(m, -1);
+  live_sec->assign(m, false);
+  int slots = 0;
+  for (int k = 0; k < m; ++k) {
+    if (!live[F + k]) continue;
+    int x, y, z;
+    chain_operands(&s[k], &x, &y, &z);
+    (*live_sec)[k] = true;
+    if (adj[cur[z]]) (*tape)[k] = slots++;
+    cur[z] = F + k;
+  }
+  return slots;
+}
+
+// Leading sections of s[0..m) that fit one run: at most kMaxChain, and a tape of at most
+// kMaxChainTape values (with the rows of 64 fields and their gradients, eight warps per SM).
+static int chain_window(int F, const adha_section* s, int m) {
+  std::vector<int> tape;
+  std::vector<bool> live;
+  int k = std::min(m, kMaxChain);
+  while (k > 1 && chain_tape(F, s, k, &tape, &live) > kMaxChainTape) k = std::max(1, k - 8);
+  return k;
+}
+
+static uint64_t chain_written(const adha_section* s, int m) {
+  uint64_t w = 0;
+  for (int k = 0; k < m; ++k) {
+    int x, y, z;
+    chain_operands(&s[k], &x, &y, &z);
+    w |= 1ull << z;
+  }
+  return w;
+}
+
+static int64_t chain_pitch(int64_t n) { return (n + 127) / 128 * 128; }
+
+// gin, gout: NULL for the forward run.
+static int run_chain(const Layout& L, void* const* ptrs, const void* const* gin, void* const* gout, const adha_section* s,
+                     int m, int64_t n, float* saved, void* stream) {
+  const bool backward = gin != nullptr;
+  ChainArgs a;
+  std::memset(&a, 0, sizeof a);
+  std::vector<int> tape;
+  std::vector<bool> live;
+  a.n_tape = chain_tape(L.F, s, m, &tape, &live);
+  const uint64_t written = chain_written(s, m);
+  uint64_t touched = written;
+  for (int k = 0; k < m; ++k) {
+    int x, y, z;
+    chain_operands(&s[k], &x, &y, &z);
+    touched |= 1ull << x | 1ull << y;
+  }
+  int row_of[kMaxFields];
+  for (int g = 0; g < L.n_groups; ++g) {
+    const auto& fields = L.groups[g];
+    bool any = false, any_w = false;
+    for (int f : fields) {
+      any = any || has(touched, f);
+      any_w = any_w || has(written, f);
+    }
+    if (!any) {
+      if (backward && gin[g] != gout[g])
+        a.copy[a.n_copy++] = ChainCopy{static_cast<const uint8_t*>(gin[g]), static_cast<uint8_t*>(gout[g]), L.stride[g]};
+      continue;
+    }
+    if (fields.size() > 1) {
+      a.wide_row[a.n_wide] = (int8_t)a.n_rows;
+      a.wide_len[a.n_wide] = (int8_t)fields.size();
+      a.wide_written[a.n_wide++] = any_w ? 1 : 0;
+    }
+    for (int f : fields) {
+      ChainRow& r = a.row[a.n_rows];
+      r.state = static_cast<uint8_t*>(ptrs[g]) + L.offset_of[f];
+      r.gin = backward ? static_cast<const uint8_t*>(gin[g]) + L.offset_of[f] : nullptr;
+      r.gout = backward ? static_cast<uint8_t*>(gout[g]) + L.offset_of[f] : nullptr;
+      r.stride = L.stride[g];
+      r.saved = has(written, f) ? __builtin_popcountll(written & ((1ull << f) - 1)) : -1;
+      row_of[f] = a.n_rows++;
+    }
+  }
+  a.n = n;
+  a.n_sec = m;
+  a.pitch = chain_pitch(n);
+  a.saved = saved;
+  auto pair = [](float v) {
+    uint32_t u;
+    std::memcpy(&u, &v, 4);
+    return (unsigned long long)u << 32 | u;
+  };
+  a.neg_zero = pair(-0.0f);
+  float tp[8] = {}, tq[8] = {};
+  tanh_coefficients(tp, tq);
+  for (int j = 0; j < 8; ++j) {
+    a.tanh_p[j] = pair(tp[j]);
+    a.tanh_q[j] = pair(tq[j]);
+  }
+  // records per lane: the most that leave 12 (forward) or 8 (backward) warps per SM
+  const int per_warp = 128 * (backward ? 2 * a.n_rows + a.n_tape : a.n_rows), warps = backward ? 8 : 12;
+  int M = 4;
+  while (M > 1 && (size_t)warps * M * per_warp > kSmemPerSM - 16 * 1024) M /= 2;
+  // few records: short chunks, so that every SM has work
+  int sms = 0;
+  if (int rc = sm_count(&sms)) return rc;
+  while (M > 1 && n < (int64_t)sms * warps * 32 * M) M /= 2;
+  a.n_chunks = (n + 32 * M - 1) / (32 * M);
+  const int row_bytes = 128 * M;
+  for (int k = 0; k < m; ++k) {
+    int x, y, z;
+    chain_operands(&s[k], &x, &y, &z);
+    a.sec[k] = ChainSec{s[k].op, row_of[x] * row_bytes, row_of[y] * row_bytes, row_of[z] * row_bytes,
+                        0.0f, 0.0f, tape[k] < 0 ? -1 : tape[k] * row_bytes, 0};
+    a.sec[k].a = s[k].fparam[0];
+    a.sec[k].b = s[k].fparam[1];
+    if (live[k]) a.live[a.n_live++] = a.sec[k];
+  }
+  const size_t smem = chain_smem_bytes(a, M, backward);
+  if (smem > (size_t)kSmemLimit) return fail(ADHA_EINVAL, "the chain run's records are too wide for a 32-record chunk");
+  int blocks = 0;
+  if (int rc = cached_occupancy(300 + 10 * M + (backward ? 1 : 0), smem, &blocks)) return rc;
+  if (blocks < 1) return fail(ADHA_ENOTIMPL, "kernel does not fit on an SM");
+  const int64_t want = (a.n_chunks + kChainThreads / 32 - 1) / (kChainThreads / 32);
+  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)sms * blocks, want));
+  const int n_saved = __builtin_popcountll(written), n_touched = __builtin_popcountll(touched);
+  // what the pass has to move: the touched fields in, the written ones out and saved; backward the
+  // gradients in and out, the saved values in, and the state back
+  const double bytes = 4.0 * (double)n * (backward ? 2 * n_touched + 2 * n_saved + (n_touched - n_saved) : n_touched + 2 * n_saved);
+  return profiled(backward ? 8 : 7, m, bytes, stream, [&] { return launch_chain(a, M, backward, grid, smem, stream); });
+}
+
 void set_fused_jit(int mode) { t_fused_jit = mode; }
 void set_reduce_accumulate(bool on) { t_reduce_accumulate = on; }
 
@@ -1268,6 +1443,54 @@ int adha_section_backward(const adha_schema* schema, int64_t n, const adha_layou
   tanh_coefficients(a.tanh_p, a.tanh_q);
   const double bytes = (double)n * (section->op == ADHA_OP_MUL ? 40.0 : 28.0);
   return profiled(2, section->op, bytes, stream, [&] { return launch_backward(a, stream); });
+}
+
+int adha_chain_plan(const adha_schema* schema, int64_t n, const adha_section* sections, int32_t n_sec, int32_t* n_run,
+                    size_t* saved_bytes) {
+  clear_error();
+  if (int rc = check_schema(schema)) return rc;
+  if (!n_run || !saved_bytes) return fail(ADHA_EINVAL, "output pointers are NULL");
+  if (n < 0) return fail(ADHA_EINVAL, "n = %lld is negative", (long long)n);
+  Layout L;   // the fields' types are all that the checks need
+  L.F = schema->n_fields;
+  for (int f = 0; f < L.F; ++f) L.dtype[f] = schema->dtype[f];
+  if (int rc = check_chain(L, sections, n_sec, n)) return rc;
+  *n_run = chain_window(L.F, sections, n_sec);
+  *saved_bytes = (size_t)__builtin_popcountll(chain_written(sections, *n_run)) * (size_t)chain_pitch(n) * 4;
+  return 0;
+}
+
+static int chain_entry(const adha_schema* schema, int64_t n, const adha_layout* layout, void* const* state,
+                       const void* const* gin, void* const* gout, bool backward, const adha_section* sections,
+                       int32_t n_sec, float* saved, adha_stream stream) {
+  Layout L;
+  if (int rc = make_layout(schema, layout, &L, "")) return rc;
+  if (n < 0) return fail(ADHA_EINVAL, "n = %lld is negative", (long long)n);
+  if (int rc = check_chain(L, sections, n_sec, n)) return rc;
+  if (chain_window(L.F, sections, n_sec) < n_sec)
+    return fail(ADHA_EINVAL, "%d sections do not fit one chain run (adha_chain_plan says how many do)", n_sec);
+  if (n == 0) return 0;
+  if (int rc = check_ptrs(reinterpret_cast<const void* const*>(state), L.n_groups, "state")) return rc;
+  if (backward) {
+    if (int rc = check_ptrs(gin, L.n_groups, "incoming gradient")) return rc;
+    if (int rc = check_ptrs(reinterpret_cast<const void* const*>(gout), L.n_groups, "gradient")) return rc;
+  }
+  if (!saved || reinterpret_cast<uintptr_t>(saved) % 16) return fail(ADHA_EINVAL, "saved buffer is NULL or not 16-byte aligned");
+  return run_chain(L, state, backward ? gin : nullptr, gout, sections, n_sec, n, saved, stream);
+}
+
+int adha_chain_forward(const adha_schema* schema, int64_t n, const adha_layout* layout, void* const* ptrs,
+                       const adha_section* sections, int32_t n_sec, float* saved, adha_stream stream) {
+  clear_error();
+  return chain_entry(schema, n, layout, ptrs, nullptr, nullptr, false, sections, n_sec, saved, stream);
+}
+
+int adha_chain_backward(const adha_schema* schema, int64_t n, const adha_layout* layout, void* const* state_ptrs,
+                        const void* const* grad_in, void* const* grad_out, const adha_section* sections, int32_t n_sec,
+                        const float* saved, adha_stream stream) {
+  clear_error();
+  return chain_entry(schema, n, layout, state_ptrs, grad_in, grad_out, true, sections, n_sec,
+                     const_cast<float*>(saved), stream);
 }
 
 int adha_profile_start(int32_t max_records) {

@@ -118,6 +118,44 @@ struct BackwardArgs {
   float tanh_p[8], tanh_q[8];
 };
 
+// A run of fp32 chain sections and its gradient in one pass each (chain.cu).  Rows are the fields of
+// every group that a section of the run touches, a group's fields consecutive.
+constexpr int kMaxChain = 128;       // sections in one run
+constexpr int kMaxChainTape = 96;    // overwritten values a run's reverse walk may need
+constexpr int kChainThreads = 64;    // small CTAs: a warp's rows take 10-30 KB, so whole CTAs waste less
+struct ChainRow {
+  uint8_t* state;        // the field in record 0
+  const uint8_t* gin;    // its gradient (backward)
+  uint8_t* gout;         // where its gradient goes (gin itself, or buffers of their own)
+  int32_t stride;        // the group's struct size; 4: the row is one contiguous array
+  int32_t saved;         // its row of `saved` if the run writes it, else -1
+};
+struct __align__(16) ChainSec {
+  int32_t op, x, y, z;   // operand rows, as byte offsets for the launch's chunk
+  float a, b;            // AXPB
+  int32_t tape;          // byte offset of the tape slot for z's value from before the section, -1 if the reverse
+                         // walk does not need it
+  int32_t pad;
+};
+struct ChainCopy {       // a group the run does not touch whose gradient goes to a buffer of its own
+  const uint8_t* src;
+  uint8_t* dst;
+  int32_t stride;
+};
+struct ChainArgs {
+  int64_t n, n_chunks;   // records; chunks counting the ragged one
+  int64_t pitch;         // floats per row of `saved`: n rounded up to whole 128-record chunks
+  float* saved;
+  unsigned long long neg_zero;   // the pair (-0, -0) (see f2_mul_alone)
+  int32_t n_rows, n_sec, n_live, n_tape, n_wide, n_copy;
+  unsigned long long tanh_p[8], tanh_q[8];   // each coefficient as a pair
+  int8_t wide_row[kMaxFields], wide_len[kMaxFields], wide_written[kMaxFields];   // groups of two or more fields
+  ChainRow row[kMaxFields];
+  ChainCopy copy[kMaxGroups];
+  ChainSec sec[kMaxChain];    // the run's sections
+  ChainSec live[kMaxChain];   // those that the backward pass runs again
+};
+
 // Plan + launch helpers shared by the entry points, the measurer and the executor.
 int remap_layouts(const Layout& S, const void* const* src_ptrs, const Layout& D, void* const* dst_ptrs, int64_t n,
                   void* stream, int* launched);
@@ -185,6 +223,9 @@ int fused_occupancy(int M, bool vec, bool km, size_t smem, int* blocks);
 // Whether a fused run holds an assign or a reduce section (they have a kernel of their own).
 inline bool fused_is_km(const FusedArgs& a) { return a.reduce_sec >= 0 || a.assign_sec >= 0; }
 int launch_backward(const BackwardArgs& a, void* stream);
+int launch_chain(const ChainArgs& a, int M, bool backward, int grid, size_t smem, void* stream);
+int chain_occupancy(int M, bool backward, size_t smem, int* blocks);
+size_t chain_smem_bytes(const ChainArgs& a, int M, bool backward);
 int remap_occupancy(int unit, size_t smem, int* blocks);
 int section_occupancy(int op, size_t smem, int* blocks);
 

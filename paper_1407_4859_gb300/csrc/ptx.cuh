@@ -52,4 +52,15 @@ __device__ __forceinline__ unsigned long long f2_add_rn(unsigned long long a, un
   return r;
 }
 
+// a * b rounded on its own, as fma(a, b, -0): ptxas contracts mul.rn.f32x2 followed by add.rn.f32x2 (or
+// sub) into one fma, whatever -fmad says (measured: equal to fmaf on 4096 of 4096 random pairs,
+// to the separate operations on 3229), so a product that is added to must not be a mul.  neg_zero
+// is the pair (-0, -0), passed through the kernel's arguments: as a literal it could be folded away.
+__device__ __forceinline__ unsigned long long f2_mul_alone(unsigned long long a, unsigned long long b,
+                                                           unsigned long long neg_zero) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(neg_zero));
+  return r;
+}
+
 }  // namespace adha
