@@ -391,10 +391,10 @@ static int cached_occupancy(int kind, size_t smem, int* blocks) {
       return 0;
     }
   }
-  // kinds: < 100 remap (direct or not), 100 + op section, 200 + 10*M + vec + 2*km fused run,
-  // 300 + 10*M + backward chain run
-  const int rc = kind < 100    ? remap_occupancy(kind, smem, blocks)
-                 : kind < 200 ? section_occupancy(kind - 100, smem, blocks)
+  // kinds: < 100 remap (direct or not), 200 + 10*M + vec + 2*km fused run, 300 + 10*M + backward chain
+  // run, 1000 + 1000*op + R + vec section
+  const int rc = kind < 100     ? remap_occupancy(kind, smem, blocks)
+                 : kind >= 1000 ? section_occupancy(kind / 1000 - 1, kind % 1000 & ~1, kind & 1, smem, blocks)
                  : kind >= 300 ? chain_occupancy((kind - 300) / 10, (kind - 300) % 10 != 0, smem, blocks)
                               : fused_occupancy((kind - 200) / 10, ((kind - 200) % 10) & 1, ((kind - 200) % 10) >> 1,
                                                 smem, blocks);
@@ -592,6 +592,17 @@ static bool reduce_walks(const Layout& L, const adha_section* s) {
   return true;
 }
 
+// Whether a staged slice keeps 16 bytes of room after each record.  Lanes read one field of
+// consecutive records, and a struct of an even number of 16-byte pieces puts those on few banks (64
+// bytes: 2 banks, 128 bytes: one).  With an odd number of pieces per staged record they spread over 8
+// (4-byte loads) or all 32 (16-byte loads).  K-Means assign of 2^24 records of 64 bytes: 604 us
+// without.
+static bool staged_room(int stride) { return stride >= 32 && stride % 32 == 0; }
+static int staged_stride(int stride) { return stride + (staged_room(stride) ? 16 : 0); }
+
+// Chunk-buffer bytes of a slice of R records `ss` apart; with `walk`, a record of room for the zeros after it.
+static int slice_bytes(int R, int ss, bool walk) { return walk ? (R * ss + ss + 15) / 16 * 16 : R * ss; }
+
 static int check_section(const Layout& L, const adha_section* s, int64_t n, bool has_save) {
   if (!s) return fail(ADHA_EINVAL, "section is NULL");
   const int F = L.F;
@@ -691,7 +702,6 @@ static int plan_section(const Layout& L, void* const* ptrs, const adha_section* 
       buffers = (it->second.second & 4) ? 1 : 2;
     }
   }
-  if (buffers != 1) buffers = 2;
   uint64_t staged = s->read_mask;
   if (s->op == ADHA_OP_MIX) staged |= s->write_mask;
   if (save) staged |= 1ull << (s->op == ADHA_OP_MUL ? s->arg[2] : s->arg[1]);
@@ -706,9 +716,41 @@ static int plan_section(const Layout& L, void* const* ptrs, const adha_section* 
   int rec = 0;
   for (int g : groups) rec += L.stride[g];
   if (s->op == ADHA_OP_GATHER) rec += 4;
-  int R = tuned_R ? std::max(32, std::min(tuned_R, 128)) : (rec > 0 ? pick_chunk(rec, 4096, 128) : 128);
-  if (R != 32 && R != 64 && R != 128) R = R < 64 ? 32 : 64;   // 96 -> 64: the kernels exist for 32, 64, 128
+  const bool walk = reduce_walks(L, s);
+  int R = 128;
+  if (tuned_R) {
+    R = std::max(32, std::min(tuned_R, 128));
+    if (R != 32 && R != 64 && R != 128) R = R < 64 ? 32 : 64;   // 96 -> 64: the kernels exist for 32, 64, 128
+  } else if (s->op == ADHA_OP_ASSIGN || walk) {
+    // long compute per chunk: two or more records per lane share the operand loads, one buffer makes
+    // room for 16 warps.  8388608 x 132 bytes, (records per chunk, buffers): assign (32,2) 332 us,
+    // (64,2) 294, (128,1) 291, (64,1) 296, one array per field (32,2) 249, (128,1) 280, (64,1) 204;
+    // reduce (32,2) 254, (64,2) 288, (128,1) 272, (64,1) 223, but 2^24 x 28 bytes (128,1) 251,
+    // (64,1) 303 and 2^24 x 64 bytes 286 and 315.
+    R = walk && rec <= 64 ? 128 : 64;
+    if (!buffers) buffers = 1;
+  } else if (s->op == ADHA_OP_GATHER) {
+    // random reads: the most warps.  2^23 particles: 126 us at 32 records, 131 at 64, 135 at 128
+    R = 32;
+  } else if (rec > 0) {
+    R = pick_chunk(rec, 4096, 128);
+    if (R == 96) R = 64;
+  }
+  if (!tuned_R) {
+    // few records: shorter chunks, so that every SM's schedulers have a warp
+    int sms = 0;
+    if (int rc = sm_count(&sms)) return rc;
+    while (R > 32 && n < (int64_t)R * sms * 4) R /= 2;
+  }
+  if (buffers != 1) buffers = 2;
+  if (n >> 36) R = 128;   // chunk numbers below 2^32 (so many records are a few bytes each: 128 of them fit)
   fill_secop(L, s, &a.s);   // before the shared-memory size, which depends on the op
+  // three fields written one after another: one of them may be an operand of a later step
+  a.alias = 0;
+  if (s->op == ADHA_OP_DRIFT || s->op == ADHA_OP_GATHER || s->op == ADHA_OP_KICK)
+    for (int w = 0; w < 3; ++w)
+      for (int k = 0; k < (s->op == ADHA_OP_DRIFT ? 6 : s->op == ADHA_OP_KICK ? 4 : 3); ++k)
+        if (k != w && s->arg[k] == s->arg[w]) a.alias = 1;
   for (;;) {
     a.n = n;
     a.R = R;
@@ -736,15 +778,17 @@ static int plan_section(const Layout& L, void* const* ptrs, const adha_section* 
       // one coalesced store stream instead of scattered partial-record stores.
       int written = 0;
       for (int f : L.groups[g]) written += has(s->write_mask, f) ? dtype_size(L.dtype[f]) : 0;
-      const bool wide = L.stride[g] > 8 && written > 0;
-      a.writeback[k] = (int8_t)(wb_mode == 1 ? 0 : wb_mode == 2 ? wide : (wide && 4 * written >= L.stride[g]));
+      // With coinciding operands every written group is, so that a later step reads what an earlier one wrote.
+      const bool wide = (L.stride[g] > 8 || a.alias) && written > 0;
+      a.writeback[k] = (int8_t)(a.alias ? wide : wb_mode == 1 ? 0 : wb_mode == 2 ? wide : (wide && 4 * written >= L.stride[g]));
       a.n_writeback += a.writeback[k];
+      a.pad[k] = staged_room(L.stride[g]) ? 1 : 0;
       for (int f : L.groups[g]) {
         a.f[f].s0 = off + L.offset_of[f];
-        a.f[f].ss = L.stride[g];
+        a.f[f].ss = staged_stride(L.stride[g]);
         a.f[f].wsm = a.writeback[k];
       }
-      off += R * L.stride[g];
+      off += slice_bytes(R, staged_stride(L.stride[g]), walk);
     }
     if (s->op == ADHA_OP_GATHER) {
       a.perm_slot = a.n_load;
@@ -757,7 +801,7 @@ static int plan_section(const Layout& L, void* const* ptrs, const adha_section* 
     a.in_bytes = off;
     a.buffers = buffers;
     a.accumulate = t_reduce_accumulate ? 1 : 0;
-    a.reduce_walk = reduce_walks(L, s) ? 1 : 0;
+    a.reduce_walk = walk ? 1 : 0;
     // vector mapping: every staged group and every written field's group is one field wide
     // (and `save`, if any, aligned for the chunk's vector stores)
     const bool vec_op = s->op == ADHA_OP_MIX || s->op == ADHA_OP_AXPB || s->op == ADHA_OP_MUL || s->op == ADHA_OP_TANH;
@@ -774,7 +818,7 @@ static int plan_section(const Layout& L, void* const* ptrs, const adha_section* 
   a.perm = s->perm;
   a.save = static_cast<uint8_t*>(save);
   int blocks = 0;
-  if (int rc = cached_occupancy(100 + s->op, plan->smem, &blocks)) return rc;
+  if (int rc = cached_occupancy(1000 + 1000 * s->op + a.R + a.vec, plan->smem, &blocks)) return rc;
   return finish_grid(a.n_chunks, blocks, &plan->grid);
 }
 
@@ -964,9 +1008,12 @@ static int plan_fused(const Layout& L, void* const* ptrs, const adha_section* s,
   if (tuned_R) R = std::max(32, std::min(tuned_R, 128));
   else if (one_field && (size_t)kWarps * 2 * 128 * rec <= (size_t)kSmemLimit / 2 - 8192) R = 128;
   else if (one_field && (size_t)kWarps * 2 * 64 * rec <= (size_t)kSmemLimit / 2 - 8192) R = 64;
+  else if (reduce_sec >= 0 || assign_sec >= 0) R = 64;   // as the sections by themselves (plan_section)
   else R = rec > 0 ? pick_chunk(rec, 4096, 128) : 128;
   if (R != 32 && R != 64 && R != 128) R = R < 64 ? 32 : 64;
   if ((reduce_sec >= 0 || assign_sec >= 0) && R > 64) R = 64;   // the assign / reduce kernels stop at 64
+  if (n >> 36) R = reduce_sec >= 0 || assign_sec >= 0 ? 64 : 128;   // chunk numbers below 2^32
+  const bool walk = reduce_sec >= 0 && reduce_walks(L, &s[reduce_sec]);
   for (;;) {
     a.n = n;
     a.R = R;
@@ -996,7 +1043,7 @@ static int plan_fused(const Layout& L, void* const* ptrs, const adha_section* s,
         a.f[f].wsm = 1;   // every write goes to the chunk buffer; written groups go back whole
       }
       vec = vec && L.groups[g].size() == 1;
-      off += R * L.stride[g];
+      off += slice_bytes(R, L.stride[g], walk);
     }
     if (perm) {
       a.perm_slot = a.n_load;
@@ -1013,7 +1060,7 @@ static int plan_fused(const Layout& L, void* const* ptrs, const adha_section* s,
     a.reduce_sec = reduce_sec;
     a.assign_sec = assign_sec;
     a.accumulate = t_reduce_accumulate ? 1 : 0;
-    a.reduce_walk = reduce_sec >= 0 && reduce_walks(L, &s[reduce_sec]) ? 1 : 0;
+    a.reduce_walk = walk ? 1 : 0;
     plan->smem = fused_smem_bytes(a);
     if (plan->smem <= (size_t)kSmemLimit) break;
     if (R <= 32) return fail(ADHA_EINVAL, "the fused run's records are too wide for a 32-record chunk");

@@ -82,9 +82,11 @@ struct FusedArgs {
   int32_t reduce_sec;           // index of the run's REDUCE section (at most one), else -1
   int32_t assign_sec;           // index of the run's first ASSIGN section (centroids staged per CTA), else -1
   int32_t accumulate;           // REDUCE: add into the result as it is (else it is zeroed before the launch)
-  int32_t reduce_walk;          // REDUCE: no feature in a one-field slice (sums cluster by cluster)
+  int32_t reduce_walk;          // REDUCE: no feature in a one-field slice (sums cluster by cluster; a record of
+                                // room follows every slice, see reduce_chunk_any)
   GroupRef load[kMaxGroups + 1];
   int8_t writeback[kMaxGroups + 1];
+  int8_t pad[kMaxGroups + 1];   // 1: 16 bytes of room after each record of staged slice k (see staged_stride)
   FieldRef f[kMaxFields];
   float tanh_p[8], tanh_q[8];
   const int32_t* perm;

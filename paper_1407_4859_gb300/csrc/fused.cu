@@ -15,26 +15,26 @@
 #include "internal.h"
 #include "ptx.cuh"
 #include "section_ops.cuh"
+#include "staging.cuh"
 
 namespace adha {
 
-// per-CTA tables at the start of shared memory: the slice table (pointers, slice ends, write-back
-// flags), then copies of the field table and of the sections' operands.  The compute loops look
+// per-CTA tables at the start of shared memory: copies of the field table and of the sections'
+// operands, then the piece table (staging.cuh).  The compute loops look
 // fields and operands up by runtime index once per field per chunk and section; from the
 // parameter space each such lookup is an indexed constant load, whose unit saturates long before
 // the memory system does, while shared-memory loads of one address broadcast to the warp.
-constexpr int kSliceTable = (16 * (kMaxGroups + 1) + 15) / 16 * 16;
 constexpr int kFieldTable = (int)sizeof(FieldRef) * kMaxFields;
 static_assert(sizeof(FieldRef) % 8 == 0 && sizeof(SecOp) % 4 == 0, "tables are copied in whole words");
 
-// Bytes of the tables for a run of n_sec sections (the chunk buffers follow, 16-byte aligned).
-__host__ __device__ constexpr int fused_table_bytes(int n_sec) {
-  return kSliceTable + kFieldTable + ((int)sizeof(SecOp) * n_sec + 15) / 16 * 16;
+// Bytes of the tables for a run of n_sec sections and n_pieces pieces per chunk (the chunk buffers
+// follow, 16-byte aligned).
+__host__ __device__ constexpr int fused_table_bytes(int n_sec, int n_pieces) {
+  return kFieldTable + ((int)sizeof(SecOp) * n_sec + 15) / 16 * 16 + n_pieces * (int)sizeof(StagePiece);
 }
 
 // After the chunk buffers: a REDUCE's two sum tables per warp (unless it walks) and its record
-// lists (see reduce_chunk_any), then an ASSIGN's centroid pair table.
-constexpr size_t kCentroidBytes = (size_t)kCentroidPairBytes;
+// lists (see reduce_chunk_any), then an ASSIGN's centroid table.
 static_assert(kReduceTableBytes % 16 == 0 && kReduceListBytes % 16 == 0, "the centroid table stays 16-byte aligned");
 
 
@@ -103,27 +103,22 @@ __device__ __forceinline__ void fused_section_record(const FusedArgs& a, const F
 template <int M, bool VEC, bool KM>
 __global__ void __launch_bounds__(kThreads) fused_kernel(const __grid_constant__ FusedArgs a) {
   extern __shared__ __align__(16) uint8_t smem[];
-  const int n_slices = a.n_load + (a.perm_slot >= 0 ? 1 : 0);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const uint8_t** sp = reinterpret_cast<const uint8_t**>(smem);
-  int* send = reinterpret_cast<int*>(smem + 8 * (kMaxGroups + 1));
-  int* wback = send + (kMaxGroups + 1);
-  const int nb = a.buffers;   // 2: the next chunk is staged while one is computed; 1: one buffer
-  uint8_t* buf0 = smem + fused_table_bytes(a.n_sec) + (size_t)warp * nb * a.in_bytes;
-  uint8_t* buf1 = buf0 + (nb - 1) * a.in_bytes;
   constexpr int R = 32 * M;
-  for (int k = tid; k < n_slices; k += kThreads) {
-    sp[k] = a.load[k].ptr;
-    send[k] = a.load[k].start + R * a.load[k].stride;
-    wback[k] = a.writeback[k];
-  }
-  FieldRef* fr = reinterpret_cast<FieldRef*>(smem + kSliceTable);
-  SecOp* secs = reinterpret_cast<SecOp*>(smem + kSliceTable + kFieldTable);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int n_pieces = stage_pieces(a, R);
+  StagePiece* tab = reinterpret_cast<StagePiece*>(smem + fused_table_bytes(a.n_sec, 0));
+  fill_pieces(a, R, n_pieces, tab, tid);
+  const int nb = a.buffers;   // 2: the next chunk is staged while one is computed; 1: one buffer
+  uint8_t* bufs = smem + fused_table_bytes(a.n_sec, n_pieces);
+  uint8_t* buf0 = bufs + (size_t)warp * nb * a.in_bytes;
+  uint8_t* buf1 = buf0 + (nb - 1) * a.in_bytes;
+  FieldRef* fr = reinterpret_cast<FieldRef*>(smem);
+  SecOp* secs = reinterpret_cast<SecOp*>(smem + kFieldTable);
   for (int k = tid; k < kMaxFields * (int)(sizeof(FieldRef) / 8); k += kThreads)
     reinterpret_cast<uint2*>(fr)[k] = reinterpret_cast<const uint2*>(a.f)[k];
   for (int k = tid; k < a.n_sec * (int)(sizeof(SecOp) / 4); k += kThreads)
     reinterpret_cast<uint32_t*>(secs)[k] = reinterpret_cast<const uint32_t*>(a.sec)[k];
-  uint8_t* extra = smem + fused_table_bytes(a.n_sec) + (size_t)kWarps * nb * a.in_bytes;
+  uint8_t* extra = bufs + (size_t)kWarps * nb * a.in_bytes;
   long long* acc = nullptr;   // REDUCE: this warp's sum tables (or register sums) and record list;
   int* idx = nullptr;         // its counts, one cluster per lane
   unsigned long long cnt_lane = 0;
@@ -133,8 +128,11 @@ __global__ void __launch_bounds__(kThreads) fused_kernel(const __grid_constant__
       acc = reinterpret_cast<long long*>(extra) + (size_t)warp * 2 * (kMaxClusters + 1) * 32;
       for (int k = lane; k < 2 * (kMaxClusters + 1) * 32; k += 32) acc[k] = 0;
       extra += kReduceTableBytes;
+    } else {
+      zero_records(a, R, buf0, lane);
+      if (nb == 2) zero_records(a, R, buf1, lane);
     }
-    idx = reinterpret_cast<int*>(extra) + warp * 32;
+    idx = reinterpret_cast<int*>(extra) + warp * kReduceList;
     extra += kReduceListBytes;
 #pragma unroll
     for (int k = 0; k < (KM ? kMaxClusters : 1); ++k) sum[k] = 0;
@@ -142,29 +140,20 @@ __global__ void __launch_bounds__(kThreads) fused_kernel(const __grid_constant__
   float* cT = nullptr;
   if (KM && a.assign_sec >= 0) {
     cT = reinterpret_cast<float*>(extra);
-    fill_centroid_pairs(a.sec[a.assign_sec], a.f, cT, tid, kThreads);
+    fill_centroids(a.sec[a.assign_sec], a.f, cT, tid, kThreads);
   }
   __syncthreads();
   ReduceLane rq{};
   if (KM && a.reduce_sec >= 0) rq = reduce_lane(secs[a.reduce_sec], fr, lane, a.reduce_walk != 0);
 
   const int64_t W = (int64_t)gridDim.x * kWarps;
-  auto stage = [&](int64_t ch, uint8_t* buf) {
-    int g = 0, start = 0;
-    for (int p = lane * 16; p < a.in_bytes; p += 512) {
-      while (p >= send[g]) start = send[g++];
-      const int64_t stride = (send[g] - start) / R;
-      cp_async16(buf + p, sp[g] + ch * (R * stride) + (p - start));
-    }
-  };
-
   int64_t c = (int64_t)blockIdx.x * kWarps + warp;
-  if (c < a.n_chunks) stage(c, buf0);
+  if (c < a.n_chunks) stage_chunk(tab, n_pieces, c, buf0, lane);
   cp_async_commit();
   for (int i = 0; c < a.n_chunks; c += W, ++i) {
     uint8_t* cur = (i & 1) ? buf1 : buf0;
     if (nb == 2) {
-      if (c + W < a.n_chunks) stage(c + W, (i & 1) ? buf0 : buf1);
+      if (c + W < a.n_chunks) stage_chunk(tab, n_pieces, c + W, (i & 1) ? buf0 : buf1, lane);
       cp_async_commit();
       cp_async_wait<1>();
     } else {
@@ -192,18 +181,10 @@ __global__ void __launch_bounds__(kThreads) fused_kernel(const __grid_constant__
       __syncwarp();   // the next section may map records to lanes the other way
     }
     // groups with written fields go back whole, 16 bytes per lane per step
-    int g = 0, start = 0;
-    for (int p = lane * 16; p < a.in_bytes; p += 512) {
-      while (p >= send[g]) start = send[g++];
-      if (wback[g]) {
-        const int64_t stride = (send[g] - start) / R;
-        *reinterpret_cast<uint4*>(const_cast<uint8_t*>(sp[g]) + c * (R * stride) + (p - start)) =
-            *reinterpret_cast<const uint4*>(cur + p);
-      }
-    }
+    unstage_chunk(tab, n_pieces, c, cur, lane);
     __syncwarp();
     if (nb == 1 && c + W < a.n_chunks) {   // one buffer: the next chunk once this one has gone back
-      stage(c + W, buf0);
+      stage_chunk(tab, n_pieces, c + W, buf0, lane);
       cp_async_commit();
     }
   }
@@ -238,9 +219,9 @@ __global__ void __launch_bounds__(kThreads) fused_kernel(const __grid_constant__
 }
 
 size_t fused_smem_bytes(const FusedArgs& a) {
-  return fused_table_bytes(a.n_sec) + (size_t)kWarps * a.buffers * a.in_bytes +
+  return fused_table_bytes(a.n_sec, stage_pieces(a, a.R)) + (size_t)kWarps * a.buffers * a.in_bytes +
          (a.reduce_sec >= 0 ? (a.reduce_walk ? 0 : kReduceTableBytes) + kReduceListBytes : 0) +
-         (a.assign_sec >= 0 ? kCentroidBytes : 0);
+         (a.assign_sec >= 0 ? (size_t)kCentroidBytes : 0);
 }
 
 template <int M, bool VEC, bool KM>

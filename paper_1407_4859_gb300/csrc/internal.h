@@ -93,11 +93,15 @@ struct SectionArgs {
   int32_t perm_slot;            // index of the staged perm slice (GATHER), else -1
   GroupRef load[kMaxGroups + 1];
   int8_t writeback[kMaxGroups + 1];   // staged slice k is written back whole after the chunk
+  int8_t pad[kMaxGroups + 1];         // 1: 16 bytes of room after each record of staged slice k (see staged_stride)
   int32_t n_writeback;
   int32_t vec;                        // 1: every accessed group is one field wide; lane = M consecutive records
   int32_t buffers;                    // chunk buffers per warp: 2 (the next chunk staged during this one) or 1
   int32_t accumulate;                 // REDUCE: add into the result as it is (else it is zeroed first)
-  int32_t reduce_walk;                // REDUCE: no feature in a one-field slice (sums cluster by cluster)
+  int32_t reduce_walk;                // REDUCE: no feature in a one-field slice (sums cluster by cluster; a record
+                                      // of room follows every slice, see reduce_chunk_any)
+  int32_t alias;                      // a field this op writes is another of its operands too: records go one
+                                      // after another through StagedRec
   FieldRef f[kMaxFields];
   float tanh_p[8], tanh_q[8];   // tanh polynomial coefficients (7 used each)
   const int32_t* perm;
@@ -227,6 +231,6 @@ int launch_chain(const ChainArgs& a, int M, bool backward, int grid, size_t smem
 int chain_occupancy(int M, bool backward, size_t smem, int* blocks);
 size_t chain_smem_bytes(const ChainArgs& a, int M, bool backward);
 int remap_occupancy(int unit, size_t smem, int* blocks);
-int section_occupancy(int op, size_t smem, int* blocks);
+int section_occupancy(int op, int R, bool vec, size_t smem, int* blocks);
 
 }  // namespace adha

@@ -17,6 +17,11 @@ __device__ __forceinline__ void cp_async16(void* sdst, const void* gsrc) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(sdst)), "l"(gsrc) : "memory");
 }
 
+// The same with the shared address already formed.
+__device__ __forceinline__ void cp_async16_at(uint32_t sdst, const void* gsrc) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sdst), "l"(gsrc) : "memory");
+}
+
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 
 // Wait until at most N of this thread's committed cp.async groups are pending.
@@ -27,7 +32,8 @@ __device__ __forceinline__ void cp_async_wait() {
 
 // Two fp32 values in one 64-bit register (low half first).  The packed instructions (sm_100 and
 // later) compute both halves in one issue slot, each an IEEE fp32 operation rounded to nearest
-// on its own (no flush to zero), so a pair gives the bits of the two scalar operations.
+// on its own (no flush to zero), so a pair gives the bits of the two scalar operations.  There is no
+// packed product here: see f2_mul_alone.
 __device__ __forceinline__ unsigned long long f2_pack(float lo, float hi) {
   unsigned long long r;
   asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
@@ -41,9 +47,9 @@ __device__ __forceinline__ unsigned long long f2_sub_rn(unsigned long long a, un
   asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
   return r;
 }
-__device__ __forceinline__ unsigned long long f2_mul_rn(unsigned long long a, unsigned long long b) {
+__device__ __forceinline__ unsigned long long f2_fma_rn(unsigned long long a, unsigned long long b, unsigned long long c) {
   unsigned long long r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
   return r;
 }
 __device__ __forceinline__ unsigned long long f2_add_rn(unsigned long long a, unsigned long long b) {

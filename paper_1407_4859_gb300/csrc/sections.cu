@@ -4,37 +4,37 @@
 //
 // The forward kernel works per warp on chunks of R = 32*M records, like remap.cu: it copies the
 // chunk's slice of every group that holds a field the section reads into its own shared buffer
-// (16-byte cp.async, one chunk ahead), computes the M records of each lane from the staged
+// (16-byte cp.async through the piece table of staging.cuh, one chunk ahead), computes the M records of each lane from the staged
 // bytes, and stores the written fields straight to global memory (a partial-record store
 // touches only the sectors of the written field).  The op is a template parameter; the layout is
 // the FieldRef table (where each field sits in the stage and in global memory).  Every floating
 // operation is an explicitly rounded-to-nearest intrinsic, so no contraction can change a bit.
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "internal.h"
 #include "ptx.cuh"
 #include "section_ops.cuh"
+#include "staging.cuh"
 
 namespace adha {
-
-// per-CTA slice table at the start of shared memory: pointers, slice ends, write-back flags
-constexpr int kSectionTable = (16 * (kMaxGroups + 1) + 15) / 16 * 16;
 
 template <int OP, int M, bool VEC>
 __global__ void __launch_bounds__(kThreads) section_kernel(const __grid_constant__ SectionArgs a) {
   extern __shared__ __align__(16) uint8_t smem[];
-  const int n_slices = a.n_load + (a.perm_slot >= 0 ? 1 : 0);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  // slice table: base pointer and byte range of each staged slice within a chunk buffer
-  const uint8_t** sp = reinterpret_cast<const uint8_t**>(smem);
-  int* send = reinterpret_cast<int*>(smem + 8 * (kMaxGroups + 1));
-  int* wback = send + (kMaxGroups + 1);
-  const int nb = a.buffers;   // 2: the next chunk is staged while one is computed; 1: one buffer
-  uint8_t* buf0 = smem + kSectionTable + (size_t)warp * nb * a.in_bytes;
-  uint8_t* buf1 = buf0 + (nb - 1) * a.in_bytes;
   constexpr int R = 32 * M;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int n_pieces = stage_pieces(a, R);
+  StagePiece* tab = reinterpret_cast<StagePiece*>(smem);
+  fill_pieces(a, R, n_pieces, tab, tid);
+  const int nb = a.buffers;   // 2: the next chunk is staged while one is computed; 1: one buffer
+  uint8_t* bufs = smem + n_pieces * sizeof(StagePiece);
+  uint8_t* buf0 = bufs + (size_t)warp * nb * a.in_bytes;
+  uint8_t* buf1 = buf0 + (nb - 1) * a.in_bytes;
+  uint8_t* extra = bufs + (size_t)kWarps * nb * a.in_bytes;
   // REDUCE: counts and (walk) sums in registers; after the chunk buffers the warp's two sum
-  // tables (not walk) and its 32-entry record list (walk)
+  // tables (not walk) and its record list (walk)
   long long* acc = nullptr;
   int* idx = nullptr;
   unsigned long long cnt = 0;   // REDUCE: lane k counts cluster k
@@ -42,49 +42,52 @@ __global__ void __launch_bounds__(kThreads) section_kernel(const __grid_constant
   ReduceLane rq{};
   if constexpr (OP == ADHA_OP_REDUCE) {
     rq = reduce_lane(a.s, a.f, lane, a.reduce_walk != 0);
-    uint8_t* extra = smem + kSectionTable + (size_t)kWarps * nb * a.in_bytes;
     if (!rq.walk) {
       acc = reinterpret_cast<long long*>(extra) + (size_t)warp * 2 * (kMaxClusters + 1) * 32;
       for (int k = lane; k < 2 * (kMaxClusters + 1) * 32; k += 32) acc[k] = 0;
       extra += kReduceTableBytes;
+    } else {
+      zero_records(a, R, buf0, lane);
+      if (nb == 2) zero_records(a, R, buf1, lane);
     }
-    idx = reinterpret_cast<int*>(extra) + warp * 32;
+    idx = reinterpret_cast<int*>(extra) + warp * kReduceList;
 #pragma unroll
     for (int k = 0; k < kMaxClusters; ++k) sum[k] = 0;
   }
-  for (int k = tid; k < n_slices; k += kThreads) {
-    sp[k] = a.load[k].ptr;
-    send[k] = a.load[k].start + R * a.load[k].stride;
-    wback[k] = a.writeback[k];
-  }
-  // ASSIGN: the centroid pair table after the chunk buffers
+  // ASSIGN: the centroid table after the chunk buffers
   float* cT = nullptr;
   if constexpr (OP == ADHA_OP_ASSIGN) {
-    cT = reinterpret_cast<float*>(smem + kSectionTable + (size_t)kWarps * nb * a.in_bytes);
-    fill_centroid_pairs(a.s, a.f, cT, tid, kThreads);
+    cT = reinterpret_cast<float*>(extra);
+    fill_centroids(a.s, a.f, cT, tid, kThreads);
+  }
+  constexpr bool kHoisted = OP != ADHA_OP_MIX && OP != ADHA_OP_ASSIGN && OP != ADHA_OP_REDUCE && !VEC;
+  constexpr int kOps = kHoisted ? kOperands<OP> : 1;
+  OpRef ref[kOps];
+  LocalOp lo;
+  if constexpr (kHoisted) {
+#pragma unroll
+    for (int k = 0; k < kOps; ++k) {
+      const FieldRef& F = a.f[a.s.arg[k]];
+      ref[k] = OpRef{F.s0 + lane * F.ss, 32 * F.ss, F.g, F.gs, F.wsm};
+      lo.arg[k] = k;
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      lo.par[k] = a.s.par[k];
+      lo.gidx[k] = a.s.gidx[k];
+    }
+    lo.gvec = a.s.gvec;
   }
   __syncthreads();
 
   const int64_t W = (int64_t)gridDim.x * kWarps;
-  // The chunk's slices are contiguous in the buffer and each a multiple of 64 bytes, so the
-  // warp walks the whole buffer in 16-byte pieces (512 bytes per step, every lane busy); piece
-  // p of slice g comes from byte (ch*R*stride_g + p - start_g) of group g.
-  auto stage = [&](int64_t ch, uint8_t* buf) {
-    int g = 0, start = 0;
-    for (int p = lane * 16; p < a.in_bytes; p += 512) {
-      while (p >= send[g]) start = send[g++];
-      const int64_t stride = (send[g] - start) / R;
-      cp_async16(buf + p, sp[g] + ch * (R * stride) + (p - start));
-    }
-  };
-
   int64_t c = (int64_t)blockIdx.x * kWarps + warp;
-  if (c < a.n_chunks) stage(c, buf0);
+  if (c < a.n_chunks) stage_chunk(tab, n_pieces, c, buf0, lane);
   cp_async_commit();
   for (int i = 0; c < a.n_chunks; c += W, ++i) {
     uint8_t* cur = (i & 1) ? buf1 : buf0;
     if (nb == 2) {
-      if (c + W < a.n_chunks) stage(c + W, (i & 1) ? buf0 : buf1);
+      if (c + W < a.n_chunks) stage_chunk(tab, n_pieces, c + W, (i & 1) ? buf0 : buf1, lane);
       cp_async_commit();
       cp_async_wait<1>();
     } else {
@@ -96,35 +99,49 @@ __global__ void __launch_bounds__(kThreads) section_kernel(const __grid_constant
       reduce_chunk_any<M>(rq, cur, lane, acc, acc + (kMaxClusters + 1) * 32, idx, sum, &cnt);
     } else if constexpr (OP == ADHA_OP_ASSIGN) {
       assign_chunk<M>(a.s, a.f, cur, i0, lane, cT);
-    } else if (OP == ADHA_OP_MIX && VEC) {
+    } else if constexpr (OP == ADHA_OP_MIX && VEC) {
       mix_chunk_vec<M>(a.s, a.f, cur, i0, lane);
-    } else if (VEC) {
+    } else if constexpr (VEC) {
       chain_chunk_vec<OP, M>(a.s, a.f, a.tanh_p, a.tanh_q, a.save, cur, i0, lane);
-    } else if (OP == ADHA_OP_MIX) {
+    } else if constexpr (OP == ADHA_OP_MIX) {
       mix_chunk<M>(a.s, a.f, cur, i0, lane);
     } else {
       const int32_t* ps = a.perm_slot >= 0 ? reinterpret_cast<const int32_t*>(cur + a.load[a.perm_slot].start) : nullptr;
+      if ((OP == ADHA_OP_DRIFT || OP == ADHA_OP_GATHER || OP == ADHA_OP_KICK) && a.alias) {
+#pragma unroll 1
+        for (int m = 0; m < M; ++m) {
+          const int r = lane + 32 * m;
+          run_record<OP>(a.s, a.f, a.tanh_p, a.tanh_q, a.save, StagedRec{a.f, cur, r, i0 + r}, i0 + r, ps ? ps[r] : 0);
+        }
+      } else {
+        unsigned long long out[M][kOps];
 #pragma unroll
-      for (int m = 0; m < M; ++m) {
-        const int r = lane + 32 * m;
-        run_record<OP>(a.s, a.f, a.tanh_p, a.tanh_q, a.save, StagedRec{a.f, cur, r, i0 + r}, i0 + r, ps ? ps[r] : 0);
+        for (int m = 0; m < M; ++m) {
+          const int r = lane + 32 * m;
+          run_record<OP>(lo, ref, a.tanh_p, a.tanh_q, a.save, HoistedRec{ref, cur, m, out[m]}, i0 + r, ps ? ps[r] : 0);
+        }
+#pragma unroll
+        for (int k = 0; k < kOps; ++k) {
+          if (!(kWrites<OP> >> k & 1)) continue;
+          using V = std::conditional_t<kWriteSize<OP> == 8, unsigned long long, uint32_t>;
+          if (ref[k].wsm) {
+#pragma unroll
+            for (int m = 0; m < M; ++m) *reinterpret_cast<V*>(cur + ref[k].s + m * ref[k].step) = (V)out[m][k];
+          } else {
+            uint8_t* q = ref[k].g + (i0 + lane) * ref[k].gs;
+#pragma unroll
+            for (int m = 0; m < M; ++m) *reinterpret_cast<V*>(q + (int64_t)(32 * m) * ref[k].gs) = (V)out[m][k];
+          }
+        }
       }
     }
     if (a.n_writeback) {   // wide written groups go back whole, 16 bytes per lane per step
       __syncwarp();
-      int g = 0, start = 0;
-      for (int p = lane * 16; p < a.in_bytes; p += 512) {
-        while (p >= send[g]) start = send[g++];
-        if (wback[g]) {
-          const int64_t stride = (send[g] - start) / R;
-          *reinterpret_cast<uint4*>(const_cast<uint8_t*>(sp[g]) + c * (R * stride) + (p - start)) =
-              *reinterpret_cast<const uint4*>(cur + p);
-        }
-      }
+      unstage_chunk(tab, n_pieces, c, cur, lane);
     }
     __syncwarp();
     if (nb == 1 && c + W < a.n_chunks) {   // one buffer: the next chunk once this one is done with it
-      stage(c + W, buf0);
+      stage_chunk(tab, n_pieces, c + W, buf0, lane);
       cp_async_commit();
     }
   }
@@ -205,10 +222,10 @@ __global__ void __launch_bounds__(kThreads) backward_kernel(const __grid_constan
 }
 
 size_t section_smem_bytes(const SectionArgs& a) {
-  // REDUCE: two (K+1) x 32 int64 tables per warp unless it walks, and a 32-entry list per warp
+  // REDUCE: two (K+1) x 32 int64 tables per warp unless it walks, and a record list per warp
   const size_t acc = a.s.op == ADHA_OP_REDUCE ? (a.reduce_walk ? 0 : kReduceTableBytes) + kReduceListBytes : 0;
-  const size_t cent = a.s.op == ADHA_OP_ASSIGN ? (size_t)kCentroidPairBytes : 0;
-  return kSectionTable + (size_t)kWarps * a.buffers * a.in_bytes + acc + cent;
+  const size_t cent = a.s.op == ADHA_OP_ASSIGN ? (size_t)kCentroidBytes : 0;
+  return (size_t)stage_pieces(a, a.R) * sizeof(StagePiece) + (size_t)kWarps * a.buffers * a.in_bytes + acc + cent;
 }
 
 template <int OP, int M, bool VEC>
@@ -239,13 +256,27 @@ static int launch_op(const SectionArgs& a, int grid, size_t smem, void* stream) 
   }
 }
 
-template <int OP>
-static int occ_op(size_t smem, int* blocks) {
-  cudaError_t e = cudaFuncSetAttribute(section_kernel<OP, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+template <int OP, int M, bool VEC>
+static int occ_om(size_t smem, int* blocks) {
+  cudaError_t e = cudaFuncSetAttribute(section_kernel<OP, M, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(section)");
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, section_kernel<OP, 1, false>, kThreads, smem);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, section_kernel<OP, M, VEC>, kThreads, smem);
   if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor(section)");
   return 0;
+}
+
+// The kernel that launch_op picks for R records per chunk.
+template <int OP>
+static int occ_op(int R, bool vec, size_t smem, int* blocks) {
+  if constexpr (kVectorOp<OP>) {
+    if (vec && R == 64) return occ_om<OP, 2, true>(smem, blocks);
+    if (vec && R == 128) return occ_om<OP, 4, true>(smem, blocks);
+  }
+  switch (R) {
+    case 32: return occ_om<OP, 1, false>(smem, blocks);
+    case 64: return occ_om<OP, 2, false>(smem, blocks);
+    default: return occ_om<OP, 4, false>(smem, blocks);
+  }
 }
 
 #define ADHA_FOR_EACH_OP(X)                                                                              \
@@ -262,9 +293,9 @@ int launch_section(const SectionArgs& a, int grid, size_t smem, void* stream) {
   }
 }
 
-int section_occupancy(int op, size_t smem, int* blocks) {
+int section_occupancy(int op, int R, bool vec, size_t smem, int* blocks) {
   switch (op) {
-#define X(o) case o: return occ_op<o>(smem, blocks);
+#define X(o) case o: return occ_op<o>(R, vec, smem, blocks);
     ADHA_FOR_EACH_OP(X)
 #undef X
     default: return fail(ADHA_EINVAL, "unknown section op %d", op);
