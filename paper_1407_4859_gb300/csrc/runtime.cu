@@ -661,7 +661,11 @@ int adha_run_program(const adha_schema* schema, int64_t n, const adha_layout* in
       return rc;
     plan->n_launches += n > 0 ? 1 : 0;
   }
-  if (back && !same_layout(cur, in)) {
+  // also when the last layout equals the input's but its groups lie elsewhere (a plan that left that
+  // layout and came back to it): identical groups at other addresses are copied
+  bool home = same_layout(cur, in);
+  for (int g = 0; g < in.n_groups && home; ++g) home = cur_p[g] == in_ptrs[g];
+  if (back && !home) {
     std::vector<void*> dp(in_ptrs, in_ptrs + in.n_groups);
     int launched = 0;
     if (int rc = remap_layouts(cur, cur_p.data(), in, dp.data(), n, stream, &launched)) return rc;
