@@ -444,8 +444,9 @@ size_t adha_measure_workspace_bytes_for(const adha_schema* schema, int64_t n, co
  * leaves that group in place, as the executor does.  With ADHA_MEASURE_AUTOTUNE
  * in flags each section is timed under every launch shape (records per chunk
  * 32, 64, 128 x field-wise or whole-group stores), and each remap from or to
- * the input layout under every choice of piece tables and chunk buffers (adha_tune_remap_pieces),
- * then under chunks of 24 to 128 records with the best of those choices;
+ * the input layout by the library's own choice of kernel, then under every choice
+ * of piece tables and chunk buffers (adha_tune_remap_pieces), then under chunks of
+ * 24 to 128 records with the best of those choices;
  * the fastest enters the table and the library's tuning cache, which later
  * launches of the same section (or pair of layouts), layout and size class use.
  * With ADHA_MEASURE_DIFFERENTIABLE (fp32 schemas whose sections are all axpb,
@@ -736,8 +737,10 @@ int adha_tune_remap_direct(int32_t mode);
  * of a chunk buffer lives in global memory (through a per-block table of the
  * pieces, or by a search over the groups) and how many input chunk buffers a
  * warp has.  0 = as tuned for the pair of layouts (adha_measure with
- * ADHA_MEASURE_AUTOTUNE), else automatic (the table for a buffer whose slices
- * average under 256 bytes; two buffers); 1..8 = forced, with bits mode - 1:
+ * ADHA_MEASURE_AUTOTUNE), else automatic: field by field with a record per lane
+ * where the layouts suit it, else through the element schedule (the table for a
+ * buffer whose slices average under 256 bytes; two buffers).  1..8 = through the
+ * schedule, with bits mode - 1:
  * bit 0 = stage the source buffer through the table, bit 1 = write the
  * destination buffer back through it, bit 2 = one input buffer (the next chunk
  * staged once the moves have read the current one) instead of two.  Every mode
@@ -749,8 +752,8 @@ int adha_tune_remap_pieces(int32_t mode);
 int adha_tune_clear(void);
 
 /* Writes the tuning cache as text ("key<TAB>records<TAB>mode" lines; section
- * keys start with S, remap keys with M and carry records 0 and the piece-table
- * bits as mode) into buf
+ * keys start with S, remap keys with M and carry records per chunk (0: by size;
+ * 1024: the library's own choice of kernel) and the piece-table bits as mode) into buf
  * (len bytes, NUL-terminated); *needed = bytes required.  buf may be NULL to
  * ask for the size.  Host only. */
 int adha_tune_export(char* buf, size_t len, size_t* needed);

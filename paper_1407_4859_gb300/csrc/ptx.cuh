@@ -22,6 +22,11 @@ __device__ __forceinline__ void cp_async16_at(uint32_t sdst, const void* gsrc) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sdst), "l"(gsrc) : "memory");
 }
 
+// A 16-byte copy of which only the first `bytes` are read (the rest of the destination is zeroed).
+__device__ __forceinline__ void cp_async16_part(uint32_t sdst, const void* gsrc, int bytes) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(sdst), "l"(gsrc), "r"(bytes) : "memory");
+}
+
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 
 // Wait until at most N of this thread's committed cp.async groups are pending.

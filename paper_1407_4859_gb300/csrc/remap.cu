@@ -122,6 +122,278 @@ size_t remap_smem_bytes(const RemapArgs& a) {
          (size_t)kWarps * ((size_t)a.buffers * ((size_t)a.in_bytes + kZeroTail) + a.out_bytes);
 }
 
+// ---------------------------------------------------------------------------------------------
+// Remap by columns: the default for a pair of layouts that has not been tuned.
+//
+// The kernel above moves a chunk element by element through a schedule (three shared-memory
+// accesses and the unpacking per element, a table of R x fields entries built by every CTA, one
+// buffer for each side).  Here a lane is a record and a step is one field of 32 records, so that a
+// field's place is one table entry for the whole chunk and the consecutive records of a one-field
+// group are one coalesced access: such groups need no buffer and no 16-byte copy loop at all.
+//   source struct -> one-field group:  shared load, global store
+//   one-field group -> destination struct:  global load, shared store (cp.async of 4 bytes into place:
+//     190 us where this takes 165; slices of the chunk staged first: 204)
+//   struct -> struct:  shared load, shared store
+// Structs move in and out in 16-byte pieces as above.  Structs of an even number of pieces are staged
+// with 16 bytes of room, or 32 records' fields would lie on a few banks.
+template <int M, bool STAGED>
+struct Columns {
+  const ColumnArgs& a;
+  const ColMove* col;
+  const ColSlice *in, *out;
+  int R, lane;
+  uint8_t *ibuf, *obuf;   // the warp's input buffers and its output buffer
+
+  __device__ __forceinline__ uint8_t* ib(int b) const { return ibuf + b * a.in_bytes; }
+  __device__ __forceinline__ bool on(int m, int cnt) const { return lane + 32 * m < cnt; }
+
+  // Places of the 16-byte pieces of `bytes` bytes of a slice: f(piece offset in memory, in the buffer).
+  template <class F>
+  __device__ __forceinline__ void pieces(const ColSlice& s, int bytes, F f) const {
+    if (s.stride & kColRoom) {
+      for (int p = lane * 16; p < bytes; p += 512) f(p, p + 16 * (int)__umulhi((unsigned)p, s.magic));
+    } else {
+      for (int p = lane * 16; p < bytes; p += 512) f(p, p);
+    }
+  }
+
+  // The chunk's source slices into buffer b.
+  template <bool WHOLE>
+  __device__ __forceinline__ void stage(int64_t ch, int b, int cnt) const {
+    const uint32_t si = smem_addr(ib(b));
+    for (int k = 0; k < a.n_in; ++k) {
+      const ColSlice s = in[k];
+      const int stride = s.stride & kColStride, bytes = cnt * stride;
+      const uint8_t* src = s.ptr + (uint64_t)(uint32_t)ch * (uint32_t)(R * stride);
+      const uint32_t dst = si + s.at;
+      pieces(s, bytes, [&](int p, int at) {
+        if (WHOLE) cp_async16_at(dst + at, src + p);
+        else cp_async16_part(dst + at, src + p, min(16, bytes - p));
+      });
+    }
+  }
+
+  template <class V, bool WHOLE>
+  __device__ __forceinline__ void column_out(int k, int end, const uint8_t* src0, int64_t i0, int cnt) const {
+    const int64_t at = (i0 + lane) * (int64_t)sizeof(V);
+#pragma unroll 4
+    for (; k < end; ++k) {
+      const ColMove t = col[k];
+      const uint8_t* src = src0 + t.off + lane * t.stride;
+      V* dst = reinterpret_cast<V*>(const_cast<uint8_t*>(t.g) + at);
+      V v[M];
+#pragma unroll
+      for (int m = 0; m < M; ++m)
+        if ((WHOLE && M > 1) || on(m, cnt)) v[m] = *reinterpret_cast<const V*>(src + m * 32 * t.stride);
+#pragma unroll
+      for (int m = 0; m < M; ++m)
+        if ((WHOLE && M > 1) || on(m, cnt)) dst[m * 32] = v[m];
+    }
+  }
+
+  // B columns at a time, so that B * M loads are in flight before the first store.
+  template <class V, bool WHOLE, int B>
+  __device__ __forceinline__ void columns_in(int k, int64_t i0, int cnt) const {
+    const int64_t at = i0 + lane;
+    V v[B][M];
+#pragma unroll
+    for (int b = 0; b < B; ++b) {
+      const V* src = reinterpret_cast<const V*>(col[k + b].g) + at;
+#pragma unroll
+      for (int m = 0; m < M; ++m)
+        if ((WHOLE && M > 1) || on(m, cnt)) v[b][m] = __ldg(src + m * 32);
+    }
+#pragma unroll
+    for (int b = 0; b < B; ++b) {
+      const ColMove t = col[k + b];
+      uint8_t* dst = obuf + t.off + lane * t.stride;
+#pragma unroll
+      for (int m = 0; m < M; ++m)
+        if ((WHOLE && M > 1) || on(m, cnt)) *reinterpret_cast<V*>(dst + m * 32 * t.stride) = v[b][m];
+    }
+  }
+  template <class V, bool WHOLE>
+  __device__ __forceinline__ void column_in(int k, int end, int64_t i0, int cnt) const {
+    for (; k + 8 <= end; k += 8) columns_in<V, WHOLE, 8>(k, i0, cnt);
+    if (k + 4 <= end) columns_in<V, WHOLE, 4>(k, i0, cnt), k += 4;
+    if (k + 2 <= end) columns_in<V, WHOLE, 2>(k, i0, cnt), k += 2;
+    if (k < end) columns_in<V, WHOLE, 1>(k, i0, cnt);
+  }
+
+  template <class V, bool WHOLE>
+  __device__ __forceinline__ void column_across(int k, int end, const uint8_t* __restrict__ src0, uint8_t* __restrict__ dst0,
+                                                int cnt) const {
+#pragma unroll 4
+    for (; k < end; ++k) {
+      const ColMove t = col[k];
+      const uint8_t* src = src0 + t.off + lane * t.stride;
+      uint8_t* dst = dst0 + t.off2 + lane * t.stride2;
+      V v[M];
+#pragma unroll
+      for (int m = 0; m < M; ++m)
+        if ((WHOLE && M > 1) || on(m, cnt)) v[m] = *reinterpret_cast<const V*>(src + m * 32 * t.stride);
+#pragma unroll
+      for (int m = 0; m < M; ++m)
+        if ((WHOLE && M > 1) || on(m, cnt)) *reinterpret_cast<V*>(dst + m * 32 * t.stride2) = v[m];
+    }
+  }
+
+  template <bool WHOLE>
+  __device__ __forceinline__ void moves(int64_t ch, int b, int cnt) const {
+    const int64_t i0 = ch * R;
+    const uint8_t* src = ib(b);
+    int k = 0, e = 0;
+    if constexpr (STAGED) {
+      e = a.cnt[0];
+      column_out<unsigned long long, WHOLE>(k, e, src, i0, cnt);
+      k = e, e += a.cnt[1];
+      column_out<uint32_t, WHOLE>(k, e, src, i0, cnt);
+      k = e, e += a.cnt[2];
+      column_out<uint16_t, WHOLE>(k, e, src, i0, cnt);
+    }
+    if constexpr (!STAGED) {
+      k = e, e += a.cnt[3];
+      column_in<unsigned long long, WHOLE>(k, e, i0, cnt);
+      k = e, e += a.cnt[4];
+      column_in<uint32_t, WHOLE>(k, e, i0, cnt);
+      return;
+    }
+    e += a.cnt[3] + a.cnt[4];
+    k = e, e += a.cnt[5];
+    column_across<unsigned long long, WHOLE>(k, e, src, obuf, cnt);
+    k = e, e += a.cnt[6];
+    column_across<uint32_t, WHOLE>(k, e, src, obuf, cnt);
+    k = e, e += a.cnt[7];
+    column_across<uint16_t, WHOLE>(k, e, src, obuf, cnt);
+  }
+
+  // The built (or carried) structs of the chunk to memory.
+  template <bool WHOLE>
+  __device__ __forceinline__ void write_out(int64_t ch, int b, int cnt) const {
+    for (int k = 0; k < a.n_out; ++k) {
+      const ColSlice s = out[k];
+      const int stride = s.stride & kColStride, bytes = cnt * stride;
+      uint8_t* dst = const_cast<uint8_t*>(s.ptr) + (uint64_t)(uint32_t)ch * (uint32_t)(R * stride);
+      const uint8_t* src = (s.stride & kColFromIn ? ib(b) : obuf) + s.at;
+      pieces(s, bytes, [&](int p, int at) {
+        if (WHOLE || p + 16 <= bytes) {
+          *reinterpret_cast<uint4*>(dst + p) = *reinterpret_cast<const uint4*>(src + at);
+        } else {
+          for (int q = 0; q < bytes - p; q += 2)
+            *reinterpret_cast<uint16_t*>(dst + p + q) = *reinterpret_cast<const uint16_t*>(src + at + q);
+        }
+      });
+    }
+  }
+};
+
+// STAGED: sources through the chunk buffer (kinds A and C); else straight from their arrays (kind B).
+template <int M, bool STAGED>
+__global__ void __launch_bounds__(kThreads, 4) column_kernel(const __grid_constant__ ColumnArgs a) {
+  extern __shared__ __align__(16) uint8_t smem[];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  int n_col = 0;
+  for (int k = 0; k < kColClasses; ++k) n_col += a.cnt[k];
+  const int nb = a.buffers;
+  ColMove* col = reinterpret_cast<ColMove*>(smem);
+  ColSlice* in = reinterpret_cast<ColSlice*>(col + n_col);
+  ColSlice* out = in + a.n_in;
+  for (int k = tid; k < n_col; k += kThreads) col[k] = a.col[k];
+  for (int k = tid; k < a.n_in; k += kThreads) in[k] = a.in[k];
+  for (int k = tid; k < a.n_out; k += kThreads) out[k] = a.out[k];
+  uint8_t* mine = reinterpret_cast<uint8_t*>(out + a.n_out) + (size_t)warp * (nb * a.in_bytes + a.out_bytes);
+  if (a.fill)
+    for (int p = lane * 16; p < a.out_bytes; p += 512)
+      *reinterpret_cast<uint4*>(mine + nb * a.in_bytes + p) = make_uint4(0, 0, 0, 0);
+  __syncthreads();
+  const int R = M == 1 ? a.R : 32 * M;
+  const Columns<M, STAGED> w{a, col, in, out, R, lane, mine, mine + nb * a.in_bytes};
+  const int64_t W = (int64_t)gridDim.x * kWarps;
+  // one input buffer: the next chunk may come in once the moves have read this one, unless groups are
+  // written from it
+  bool early = nb == 1;
+  for (int k = 0; k < a.n_out; ++k) early = early && !(out[k].stride & kColFromIn);
+
+  int64_t c = (int64_t)blockIdx.x * kWarps + warp;
+  if (c < a.n_chunks) w.template stage<true>(c, 0, R);
+  cp_async_commit();
+  for (int i = 0; c < a.n_chunks; c += W, i ^= nb - 1) {
+    const bool more = c + W < a.n_chunks;
+    if (nb == 2) {
+      if (more) w.template stage<true>(c + W, i ^ 1, R);
+      cp_async_commit();
+      cp_async_wait<1>();
+    } else {
+      cp_async_wait<0>();
+    }
+    __syncwarp();
+    w.template moves<true>(c, i, R);
+    __syncwarp();
+    if (early && more) {
+      w.template stage<true>(c + W, 0, R);
+      cp_async_commit();
+    }
+    w.template write_out<true>(c, i, R);
+    __syncwarp();
+    if (nb == 1 && !early && more) {
+      w.template stage<true>(c + W, 0, R);
+      cp_async_commit();
+    }
+  }
+  // fewer than R records at the end: the warp whose next chunk would be n_chunks
+  const int rest = (int)(a.n - a.n_chunks * R);
+  if (c == a.n_chunks && rest > 0) {
+    cp_async_wait<0>();
+    __syncwarp();
+    w.template stage<false>(c, 0, rest);
+    cp_async_commit();
+    cp_async_wait<0>();
+    __syncwarp();
+    w.template moves<false>(c, 0, rest);
+    __syncwarp();
+    w.template write_out<false>(c, 0, rest);
+  }
+  cp_async_wait<0>();
+}
+
+size_t columns_smem_bytes(const ColumnArgs& a) {
+  int n_col = 0;
+  for (int k = 0; k < kColClasses; ++k) n_col += a.cnt[k];
+  return (size_t)(n_col + a.n_in + a.n_out) * 16 + (size_t)kWarps * ((size_t)a.buffers * a.in_bytes + a.out_bytes);
+}
+
+template <int M, bool STAGED>
+static int launch_c(const ColumnArgs& a, int grid, size_t smem, void* stream) {
+  cudaError_t e = cudaFuncSetAttribute(column_kernel<M, STAGED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(columns)");
+  column_kernel<M, STAGED><<<grid, kThreads, smem, (cudaStream_t)stream>>>(a);
+  e = cudaGetLastError();
+  if (e != cudaSuccess) return cuda_fail(e, "column remap launch");
+  return 0;
+}
+
+int launch_columns(const ColumnArgs& a, int grid, size_t smem, void* stream) {
+  if (a.cnt[3] + a.cnt[4] > 0)
+    return a.R == 64 ? launch_c<2, false>(a, grid, smem, stream) : launch_c<1, false>(a, grid, smem, stream);
+  return a.R == 128  ? launch_c<4, true>(a, grid, smem, stream)
+         : a.R == 64 ? launch_c<2, true>(a, grid, smem, stream)
+                     : launch_c<1, true>(a, grid, smem, stream);
+}
+
+template <int M, bool STAGED>
+static int occ_c(size_t smem, int* blocks) {
+  cudaError_t e = cudaFuncSetAttribute(column_kernel<M, STAGED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(columns)");
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, column_kernel<M, STAGED>, kThreads, smem);
+  if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor(columns)");
+  return 0;
+}
+
+int columns_occupancy(int R, bool staged, size_t smem, int* blocks) {
+  if (!staged) return R == 64 ? occ_c<2, false>(smem, blocks) : occ_c<1, false>(smem, blocks);
+  return R == 128 ? occ_c<4, true>(smem, blocks) : R == 64 ? occ_c<2, true>(smem, blocks) : occ_c<1, true>(smem, blocks);
+}
+
 template <bool DIRECT>
 static int launch_d(const RemapArgs& a, int grid, size_t smem, void* stream) {
   cudaError_t e = cudaFuncSetAttribute(remap_kernel<DIRECT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

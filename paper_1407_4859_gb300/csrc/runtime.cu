@@ -207,9 +207,15 @@ int adha_measure(const adha_schema* schema, int64_t n, const adha_layout* in_lay
                         bool tune, double* ns) {
     auto run = [&] { return remap_layouts(S, sp.data(), D, const_cast<void**>(dp.data()), n, stream, nullptr); };
     if (!tune || !(flags & ADHA_MEASURE_AUTOTUNE)) return time_ns(timer, stream, reps, run, ns);
+    // the library's own choice first (without the tuning of an earlier call), then by the schedule with
+    // piece tables x one or two chunk buffers per warp
+    const std::string key = remap_tuning_key(S, D, n);
+    tuning_store(key, kOwnChoice, 0);
+    double own = 0;
+    if (const int e = time_ns(timer, stream, reps, run, &own)) return e;
     double best = -1, t = 0;
     int bits = 0, bestR = 0;
-    for (int m = 1; m <= 8; ++m) {   // piece tables x one or two chunk buffers per warp
+    for (int m = 1; m <= 8; ++m) {
       set_remap_pieces(m);
       const int e = time_ns(timer, stream, reps, run, &t);
       set_remap_pieces(0);
@@ -233,8 +239,8 @@ int adha_measure(const adha_schema* schema, int64_t n, const adha_layout* in_lay
         bestR = R;
       }
     }
-    tuning_store(remap_tuning_key(S, D, n), bestR, bits);
-    *ns = best;
+    if (best < own) tuning_store(key, bestR, bits);
+    *ns = std::min(best, own);
     return 0;
   };
   for (int a = 0; a < L && !rc; ++a) {
