@@ -537,7 +537,7 @@ typedef struct adha_batched adha_batched;
  * batching form of the paper's remap, Section 2): validates every array (rules
  * of adha_remap), plans each one (chunk size, element schedule) and lays out
  * the descriptors the kernel reads.  The kernel's warps work alone: each takes
- * work units of about 1024 records of one array by an atomic ticket (largest
+ * work units of up to 1024 records of one array by an atomic ticket (largest
  * array first) and keeps its current array's tables in its own region of
  * shared memory.  The region is set here: the number of CTAs per SM (1 to 8,
  * as registers allow) whose regions hold every array's chunk buffers (chunks

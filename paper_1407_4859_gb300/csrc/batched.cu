@@ -2,11 +2,11 @@
 // paper's remap edge, Section 2).
 //
 // Every array (its own schema, record count and source/destination layouts) is cut into chunks
-// of R_a records, and its chunks into work units of about 1024 records.  Each warp works alone:
+// of R_a records, and its chunks into work units of up to 1024 records.  Each warp works alone:
 // it takes the next unit with one 64-bit atomic ticket (in the descriptor region, zeroed before
 // every launch), finds the unit's array by a 32-way search over the arrays' first units (one
 // ballot per level), and, when the array differs from its last one, copies that array's header,
-// group table and element schedule (built on the host when the batch is prepared) into its own
+// group table and element schedule (built on the device when the batch is placed) into its own
 // region of shared memory.  It then runs the cp.async pipeline of remap.cu over the unit's
 // consecutive chunks: stage the source slices with 16-byte copies, assemble the destination
 // records one move per lane per step, write them back with 16-byte stores.  With one input
@@ -30,7 +30,8 @@
 
 namespace adha {
 
-constexpr int kUnitRecords = 1024;   // records of one work unit (whole chunks, at least one)
+constexpr int kUnitRecords = 1024;   // most records of one work unit (whole chunks, at least one)
+constexpr int kUnitsPerWarp = 4;     // units shrink to about this many per resident warp (see adha_batched_create)
 constexpr int kHeaderBytes = 128;    // a warp region starts with the header of its current array
 constexpr int kMaxBatchedCtas = 8;   // CTAs per SM tried (8 x 8 warps = 64 warps, the SM's limit)
 
@@ -44,6 +45,8 @@ struct BatchHeader {
   int32_t chunks_per_unit;
   int32_t sched_off, buf_off;    // offsets in a warp region: the schedule, the first chunk buffer
   int32_t sched_bytes;
+  int8_t cls_order[8];           // schedule order per move class
+  int32_t pad[2];
 };
 static_assert(sizeof(BatchHeader) <= kHeaderBytes && sizeof(BatchHeader) % 16 == 0, "header is copied in words");
 static_assert(sizeof(GroupRef) == 16, "group table is copied in 16-byte words");
@@ -60,6 +63,20 @@ struct BatchParams {
   int32_t buffers;               // input chunk buffers per warp: 2 (the next chunk staged during this one) or 1
   int64_t total_units;
 };
+
+// The arrays' element schedules, one CTA per array.  Built here and not on the host: 32 arrays of up to
+// 16384 records took 118 of 273 us of planning, and 100 KB more to copy.
+__global__ void __launch_bounds__(kThreads) schedule_kernel(const BatchHeader* headers, const GroupRef* groups,
+                                                            const Move* moves, uint8_t* sched) {
+  const BatchHeader& h = headers[blockIdx.x];
+  const GroupRef* src = groups + h.group0;
+  int32_t order[kMoveClasses];
+  for (int c = 0; c < kMoveClasses; ++c) order[c] = h.cls_order[c];
+  uint32_t* out = reinterpret_cast<uint32_t*>(sched + h.sched0);
+  const int n = h.R * h.n_moves;
+  for (int t = threadIdx.x; t < h.sched_bytes / 4; t += kThreads)
+    out[t] = t < n ? schedule_entry(t, h.R, h.cls_count, order, moves + h.move0, src, src + h.n_src, h.in_bytes) : 0u;
+}
 
 // Last array a with prefix[a] <= u: a 32-way search, one ballot per level (prefix[0] = 0 <= u,
 // so lane 0 always qualifies and the answer stays inside [lo, lo + span)).
@@ -160,7 +177,8 @@ using namespace adha;
 
 struct adha_batched {
   int32_t n_arrays = 0;            // arrays listed for the kernel (those with bytes to move)
-  std::vector<uint8_t> image;      // descriptor region as it is copied to the workspace
+  std::vector<uint8_t> image;      // descriptor region as it is copied to the workspace (its work ticket is zero)
+  size_t total = 0;                // workspace bytes: the image, then the schedules (built on the device)
   size_t off_headers = 0, off_groups = 0, off_moves = 0, off_sched = 0, off_prefix = 0;
   int64_t total_units = 0;
   int32_t region = 0;              // shared bytes per warp
@@ -195,8 +213,21 @@ static BatchParams params_for(const adha_batched* b, void* ws) {
   return p;
 }
 
-static int launch_batched(const adha_batched* b, void* ws, void* stream) {
-  cudaError_t e = cudaMemsetAsync(ws, 0, sizeof(unsigned long long), (cudaStream_t)stream);
+// The image into the workspace and the schedules built there.
+static int place_batched(const adha_batched* b, void* ws, void* stream) {
+  cudaError_t e = cudaMemcpyAsync(ws, b->image.data(), b->image.size(), cudaMemcpyHostToDevice, (cudaStream_t)stream);
+  if (e != cudaSuccess) return cuda_fail(e, "copy of the batched descriptors");
+  if (b->n_arrays == 0) return 0;
+  const BatchParams p = params_for(b, ws);
+  schedule_kernel<<<b->n_arrays, kThreads, 0, (cudaStream_t)stream>>>(p.headers, p.groups, p.moves, const_cast<uint8_t*>(p.sched));
+  e = cudaGetLastError();
+  return e == cudaSuccess ? 0 : cuda_fail(e, "batched schedule launch");
+}
+
+// zeroed: the work ticket is (the image has just been copied).
+static int launch_batched(const adha_batched* b, void* ws, void* stream, bool zeroed = false) {
+  cudaError_t e = cudaSuccess;
+  if (!zeroed) e = cudaMemsetAsync(ws, 0, sizeof(unsigned long long), (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync(ticket)");
   if (b->total_units == 0) return 0;
   auto* k = b->direct ? batched_kernel<true> : batched_kernel<false>;
@@ -402,8 +433,15 @@ int adha_batched_create(int32_t n_arrays, const adha_remap_desc* descs, int32_t 
   std::vector<BatchHeader> headers;
   std::vector<GroupRef> groups;
   std::vector<Move> moves;
-  std::vector<uint32_t> sched;
   std::vector<int64_t> prefix;
+  size_t sched_bytes = 0;
+  // Records per work unit: 1024 (a warp changes arrays, and copies their tables, once per unit), fewer
+  // where warps would get less than four.  Kernel us, always 1024 -> this: 32 arrays of 256..16384
+  // records 202 -> 21, 64 of 4096..262144 284 -> 165 (one unit per warp 206, two 175, eight 167), 256
+  // of 1024..131072 292 -> 255.
+  int64_t records = 0;
+  for (int k : order) records += plans[k].n;
+  const int unit = (int)std::max<int64_t>(32, std::min<int64_t>(kUnitRecords, records / ((int64_t)sms * best_k * kWarps * kUnitsPerWarp)));
   int64_t units = 0;
   double bytes = 0;
   bool direct = false;
@@ -430,21 +468,19 @@ int adha_batched_create(int32_t n_arrays, const adha_remap_desc* descs, int32_t 
     for (int c = 0; c < kMoveClasses; ++c) h.cls_count[c] = a.cls_count[c];
     h.group0 = (int32_t)groups.size();
     h.move0 = (int32_t)moves.size();
-    h.chunks_per_unit = std::max(1, kUnitRecords / a.R);
+    h.chunks_per_unit = std::max(1, unit / a.R);
     h.sched_bytes = al16(a.R * a.n_moves * 4);
     h.sched_off = kHeaderBytes + (a.n_src + a.n_dst) * (int)sizeof(GroupRef);
     h.buf_off = h.sched_off + h.sched_bytes;
-    h.sched0 = (int64_t)sched.size() * 4;
+    h.sched0 = (int64_t)sched_bytes;
+    sched_bytes += h.sched_bytes;
+    for (int c = 0; c < kMoveClasses; ++c) h.cls_order[c] = (int8_t)a.cls_order[c];
     h.unit0 = units;
     prefix.push_back(units);
     units += (h.n_chunks + h.chunks_per_unit - 1) / h.chunks_per_unit;
     for (int g = 0; g < a.n_src; ++g) groups.push_back(a.src[g]);
     for (int g = 0; g < a.n_dst; ++g) groups.push_back(a.dst[g]);
     moves.insert(moves.end(), a.move, a.move + a.n_moves);
-    const size_t s0 = sched.size();
-    sched.resize(s0 + h.sched_bytes / 4, 0u);
-    for (int t = 0; t < a.R * a.n_moves; ++t)
-      sched[s0 + t] = schedule_entry(t, a.R, a.cls_count, a.cls_order, a.move, a.src, a.dst, a.in_bytes);
     direct = direct || (a.cls_count[0] + a.cls_count[1] + a.cls_count[2] > 0);
     bytes += ap.moved;
     headers.push_back(h);
@@ -463,13 +499,13 @@ int adha_batched_create(int32_t n_arrays, const adha_remap_desc* descs, int32_t 
   b->off_headers = al256(sizeof(unsigned long long));
   b->off_groups = b->off_headers + al256(std::max<size_t>(1, headers.size()) * sizeof(BatchHeader));
   b->off_moves = b->off_groups + al256(std::max<size_t>(1, groups.size()) * sizeof(GroupRef));
-  b->off_sched = b->off_moves + al256(std::max<size_t>(1, moves.size()) * sizeof(Move));
-  b->off_prefix = b->off_sched + al256(std::max<size_t>(1, sched.size()) * 4);
+  b->off_prefix = b->off_moves + al256(std::max<size_t>(1, moves.size()) * sizeof(Move));
   b->image.assign(b->off_prefix + al256(prefix.size() * sizeof(int64_t)), 0);
+  b->off_sched = b->image.size();
+  b->total = b->off_sched + al256(std::max<size_t>(4, sched_bytes));
   if (!headers.empty()) std::memcpy(b->image.data() + b->off_headers, headers.data(), headers.size() * sizeof(BatchHeader));
   if (!groups.empty()) std::memcpy(b->image.data() + b->off_groups, groups.data(), groups.size() * sizeof(GroupRef));
   if (!moves.empty()) std::memcpy(b->image.data() + b->off_moves, moves.data(), moves.size() * sizeof(Move));
-  if (!sched.empty()) std::memcpy(b->image.data() + b->off_sched, sched.data(), sched.size() * 4);
   std::memcpy(b->image.data() + b->off_prefix, prefix.data(), prefix.size() * sizeof(int64_t));
   b->smem = (size_t)kWarps * best_region;
   int per_sm = 0;
@@ -486,16 +522,15 @@ int adha_batched_create(int32_t n_arrays, const adha_remap_desc* descs, int32_t 
   return 0;
 }
 
-size_t adha_batched_workspace_bytes(const adha_batched* b) { return b ? b->image.size() : 0; }
+size_t adha_batched_workspace_bytes(const adha_batched* b) { return b ? b->total : 0; }
 
 int adha_batched_upload(const adha_batched* b, void* workspace, size_t ws_bytes, adha_stream stream) {
   clear_error();
   if (!b || !workspace) return fail(ADHA_EINVAL, "NULL batched plan or workspace");
-  if (ws_bytes < b->image.size()) return fail(ADHA_ENOMEM, "workspace has %zu bytes, needs %zu", ws_bytes, b->image.size());
+  if (ws_bytes < b->total) return fail(ADHA_ENOMEM, "workspace has %zu bytes, needs %zu", ws_bytes, b->total);
   if (reinterpret_cast<uintptr_t>(workspace) % 256) return fail(ADHA_EINVAL, "workspace is not 256-byte aligned");
-  cudaError_t e = cudaMemcpyAsync(workspace, b->image.data(), b->image.size(), cudaMemcpyHostToDevice, (cudaStream_t)stream);
-  if (e != cudaSuccess) return cuda_fail(e, "upload of the batched descriptors");
-  e = cudaStreamSynchronize((cudaStream_t)stream);
+  if (int rc = place_batched(b, workspace, stream)) return rc;
+  const cudaError_t e = cudaStreamSynchronize((cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize(upload)");
   return 0;
 }
@@ -503,6 +538,12 @@ int adha_batched_upload(const adha_batched* b, void* workspace, size_t ws_bytes,
 static int batched_fn(const void* ctx) {
   const auto* c = static_cast<const std::pair<const adha_batched*, std::pair<void*, void*>>*>(ctx);
   return launch_batched(c->first, c->second.first, c->second.second);
+}
+
+// After place_batched: the ticket is zero.
+static int placed_fn(const void* ctx) {
+  const auto* c = static_cast<const std::pair<const adha_batched*, std::pair<void*, void*>>*>(ctx);
+  return launch_batched(c->first, c->second.first, c->second.second, true);
 }
 
 int adha_batched_launch(const adha_batched* b, void* workspace, adha_stream stream) {
@@ -606,7 +647,7 @@ int adha_workspace_bytes(int32_t n_arrays, const adha_remap_desc* descs, size_t*
   if (!bytes) return fail(ADHA_EINVAL, "bytes is NULL");
   adha_batched* b = nullptr;
   if (int rc = adha_batched_create(n_arrays, descs, 0, nullptr, &b)) return rc;
-  *bytes = b->image.size();
+  *bytes = b->total;
   adha_batched_destroy(b);
   return 0;
 }
@@ -619,18 +660,14 @@ int adha_remap_batched(int32_t n_arrays, const adha_remap_desc* descs, void* wor
   if (int rc = reject_capture(stream)) return rc;
   adha_batched* b = nullptr;
   if (int rc = adha_batched_create(n_arrays, descs, 0, stream, &b)) return rc;
-  if (ws_bytes < b->image.size()) {
-    const size_t need = b->image.size();
+  if (ws_bytes < b->total) {
+    const size_t need = b->total;
     adha_batched_destroy(b);
     return fail(ADHA_ENOMEM, "workspace has %zu bytes, the batch needs %zu (adha_workspace_bytes)", ws_bytes, need);
   }
-  cudaError_t e = cudaMemcpyAsync(workspace, b->image.data(), b->image.size(), cudaMemcpyHostToDevice, (cudaStream_t)stream);
-  if (e != cudaSuccess) {
-    adha_batched_destroy(b);
-    return cuda_fail(e, "copy of the batched descriptors into the workspace");
-  }
   const std::pair<const adha_batched*, std::pair<void*, void*>> ctx{b, {workspace, stream}};
-  const int rc = profiled_launch(3, 3, b->bytes, stream, batched_fn, &ctx);
+  int rc = place_batched(b, workspace, stream);
+  if (!rc) rc = profiled_launch(3, 3, b->bytes, stream, placed_fn, &ctx);
   adha_batched_destroy(b);
   return rc;
 }
@@ -680,7 +717,7 @@ extern "C" int adha_remap_batched_noalloc(int32_t n_arrays, const adha_remap_des
   if (int rc = reject_capture(stream)) return rc;
   adha_batched* b = nullptr;
   if (int rc = adha_batched_create(n_arrays, descs, 0, stream, &b)) return rc;
-  const size_t need = b->image.size();
+  const size_t need = b->total;
   if (need > (size_t)ADHA_NOALLOC_SCRATCH_BYTES) {
     adha_batched_destroy(b);
     return fail(ADHA_EINVAL, "this batch needs %zu bytes of descriptors; the allocation-free entry point holds at most %u",
@@ -692,14 +729,11 @@ extern "C" int adha_remap_batched_noalloc(int32_t n_arrays, const adha_remap_des
     std::lock_guard<std::mutex> lk(g_noalloc_mu);
     void* scratch = nullptr;
     rc = noalloc_scratch(&scratch);
-    if (!rc) {
-      // pageable source: the bytes are staged before the call returns, so the host image can go
-      const cudaError_t e = cudaMemcpyAsync(scratch, b->image.data(), need, cudaMemcpyHostToDevice, (cudaStream_t)stream);
-      if (e != cudaSuccess) rc = cuda_fail(e, "copy of the batched descriptors into the scratch array");
-    }
+    // pageable source: the bytes are staged before the call returns, so the host image can go
+    if (!rc) rc = place_batched(b, scratch, stream);
     if (!rc) {
       const std::pair<const adha_batched*, std::pair<void*, void*>> ctx{b, {scratch, stream}};
-      rc = profiled_launch(3, 2, b->bytes, stream, batched_fn, &ctx);
+      rc = profiled_launch(3, 2, b->bytes, stream, placed_fn, &ctx);
     }
   }
   adha_batched_destroy(b);

@@ -262,6 +262,14 @@ static std::string remap_key(const Layout& S, const Layout& D, int64_t n) {
   return "M" + layout_code(S) + ">" + layout_code(D) + size_class(n);
 }
 
+// Whether the cache holds any remap entry: the key of a pair of layouts, a microsecond or two of text, is
+// built only then.
+static bool any_remap_tuned() {
+  std::lock_guard<std::mutex> lk(g_tune_mu);
+  const auto it = g_tune.lower_bound("M");
+  return it != g_tune.end() && it->first[0] == 'M';
+}
+
 std::string tuning_key(const Layout& L, const adha_section* s, int64_t n, bool save) { return section_key(L, s, n, save); }
 std::string remap_tuning_key(const Layout& S, const Layout& D, int64_t n) { return remap_key(S, D, n); }
 
@@ -500,7 +508,7 @@ static int plan_remap(const Layout& S, const void* const* src_ptrs, const Layout
   for (int j : need) src_rec += S.stride[j];
   for (int d : build) dst_rec += D.stride[d];
   int tuned_pieces = -1, tuned_R = 0;
-  if (!t_remap_pieces || !t_tile_override) {
+  if ((!t_remap_pieces || !t_tile_override) && any_remap_tuned()) {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_tune.find(remap_key(S, D, n));
     if (it != g_tune.end() && it->second.first != kOwnChoice) {
@@ -988,9 +996,8 @@ static double section_bytes(const Layout& L, const adha_section* s, int64_t n, b
 // Whether the schedule was tuned to be the faster kernel for this pair of layouts (the key is built only
 // when some remap is tuned).
 static bool remap_tuned(const Layout& S, const Layout& D, int64_t n) {
+  if (!any_remap_tuned()) return false;
   std::lock_guard<std::mutex> lk(g_tune_mu);
-  const auto it = g_tune.lower_bound("M");
-  if (it == g_tune.end() || it->first[0] != 'M') return false;
   const auto f = g_tune.find(remap_key(S, D, n));
   return f != g_tune.end() && f->second.first != kOwnChoice;
 }
