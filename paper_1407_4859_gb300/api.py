@@ -4,6 +4,7 @@ PyTorch provides device memory and streams only; every byte the library moves or
 moved or computed by its CUDA kernels.  Function names follow the C ABI (adha_remap, ...).
 """
 import ctypes
+import struct
 
 import torch
 
@@ -25,6 +26,7 @@ class Schema:
         self.dtypes = [int(d) for d in dtypes]
         self._arr = _i32_array(self.dtypes)
         self.c = adha_schema(len(self.dtypes), self._arr)
+        self.address = ctypes.addressof(self.c)
 
     @property
     def F(self):
@@ -39,6 +41,7 @@ class Layout:
         self._len = _i32_array([len(g) for g in self.groups])
         self._fields = _i32_array([f for g in self.groups for f in g])
         self.c = adha_layout(len(self.groups), self._len, self._fields)
+        self.address = ctypes.addressof(self.c)
 
     def key(self):
         return tuple(tuple(g) for g in self.groups)
@@ -74,15 +77,18 @@ def adha_layout_strides(schema, layout):
     return list(st), list(off)
 
 
+def _addresses(bufs):
+    return [b.data_ptr() if isinstance(b, torch.Tensor) else int(b) for b in bufs]
+
+
 def _ptrs(bufs):
-    arr = (ctypes.c_void_p * max(1, len(bufs)))()
-    for k, b in enumerate(bufs):
-        arr[k] = b.data_ptr() if isinstance(b, torch.Tensor) else int(b)
-    return arr
+    return (ctypes.c_void_p * max(1, len(bufs)))(*_addresses(bufs))
 
 
 def _stream_ptr(stream):
     if stream is None:
+        if torch.cuda.is_initialized():   # the current stream's handle without a Stream object around it
+            return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()))
         stream = torch.cuda.current_stream()
     return ctypes.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
 
@@ -497,10 +503,9 @@ def _fix_plan(plan, fixed, windows):
     plan.fixed = 0
     if fixed is not None:
         plan.fixed = 1
-        for k, l in enumerate(fixed):
-            plan.layout_of_section[k] = int(l)
-        for k in range(len(fixed)):
-            plan.window_len[k] = int(windows[k]) if windows is not None else 0
+        S = len(fixed)
+        plan.layout_of_section[:S] = [int(l) for l in fixed]
+        plan.window_len[:S] = [int(w) for w in windows[:S]] if windows is not None else [0] * S
 
 
 def adha_run_program(schema, n, in_layout, in_bufs, sections, candidates, costs=None, opts=None, workspace=None,
@@ -597,14 +602,19 @@ ADHA_BATCHED_TWO_BUFFERS = 2
 def remap_descs(arrays):
     """(adha_remap_desc array, objects to keep alive) for a list of array dicts with keys schema,
     n, src, src_bufs, dst, dst_bufs."""
-    keep = []
     descs = (_lib.adha_remap_desc * max(1, len(arrays)))()
-    for k, a in enumerate(arrays):
-        sp, dp = _ptrs(a["src_bufs"]), _ptrs(a["dst_bufs"])
-        keep += [a["schema"], a["src"], a["dst"], sp, dp]
-        descs[k] = _lib.adha_remap_desc(ctypes.pointer(a["schema"].c), int(a["n"]), ctypes.pointer(a["src"].c),
-                                        sp, ctypes.pointer(a["dst"].c), dp)
-    return descs, keep
+    size = ctypes.sizeof(_lib.adha_remap_desc)
+    addresses, rows = [], []
+    for a in arrays:   # every buffer's address, in one array that the descriptors point into
+        first = len(addresses)
+        addresses += _addresses(a["src_bufs"])
+        rows.append((a["schema"], int(a["n"]), a["src"], first, a["dst"], len(addresses)))
+        addresses += _addresses(a["dst_bufs"])
+    ptrs = (ctypes.c_void_p * max(1, len(addresses)))(*addresses)
+    at = ctypes.addressof(ptrs)
+    for k, (schema, n, src, s, dst, d) in enumerate(rows):   # the fields of an adha_remap_desc, in order
+        struct.pack_into("PqPPPP", descs, k * size, schema.address, n, src.address, at + 8 * s, dst.address, at + 8 * d)
+    return descs, [rows, ptrs]
 
 
 def adha_workspace_bytes(arrays):

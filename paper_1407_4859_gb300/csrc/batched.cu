@@ -231,8 +231,7 @@ static int launch_batched(const adha_batched* b, void* ws, void* stream, bool ze
   if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync(ticket)");
   if (b->total_units == 0) return 0;
   auto* k = b->direct ? batched_kernel<true> : batched_kernel<false>;
-  e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b->smem);
-  if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(batched)");
+  if (int rc = allow_smem(reinterpret_cast<const void*>(k), b->smem, "cudaFuncSetAttribute(batched)")) return rc;
   k<<<b->grid, kThreads, b->smem, (cudaStream_t)stream>>>(params_for(b, ws));
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "batched kernel launch");
@@ -293,7 +292,7 @@ static int tune_chunk(const Layout& S, const void* const* sp, const Layout& D, v
     const int R = 32 << (trial >> 1), direct = trial & 1;
     RemapArgs a;
     bool empty = false;
-    rc = remap_plan_args(S, sp, D, dp, n, R, direct, &a, &empty);
+    rc = remap_plan_args(S, sp, D, dp, n, R, direct, false, &a, &empty);
     if (rc || empty) break;
     if (a.R != R) continue;   // too wide for this chunk in the single-array kernel
     rc = time_ms(R, direct, &ms);
@@ -352,7 +351,7 @@ int adha_batched_create(int32_t n_arrays, const adha_remap_desc* descs, int32_t 
     if (d.n == 0) continue;
     int R = 0, direct = 0;
     if (flags & ADHA_BATCHED_AUTOTUNE) rc = tune_chunk(ap.S, d.src_ptrs, ap.D, d.dst_ptrs, d.n, stream, &R, &direct);
-    if (!rc) rc = remap_plan_args(ap.S, d.src_ptrs, ap.D, d.dst_ptrs, d.n, R ? R : batch_chunk(ap.S, ap.D), direct, &ap.a,
+    if (!rc) rc = remap_plan_args(ap.S, d.src_ptrs, ap.D, d.dst_ptrs, d.n, R ? R : batch_chunk(ap.S, ap.D), direct, false, &ap.a,
                                   &ap.empty);
     if (rc) return rc;
     ap.R0 = ap.a.R;
@@ -451,8 +450,10 @@ int adha_batched_create(int32_t n_arrays, const adha_remap_desc* descs, int32_t 
     RemapArgs& a = ap.a;
     if (R != a.R) {
       bool empty = false;
-      if (int rc = remap_plan_args(ap.S, ap.sp, ap.D, ap.dp, ap.n, R, ap.direct, &a, &empty)) return rc;
+      if (int rc = remap_plan_args(ap.S, ap.sp, ap.D, ap.dp, ap.n, R, ap.direct, true, &a, &empty)) return rc;
       if (a.R != R) return fail(ADHA_ENOTIMPL, "batched remap: array %d cannot use %d-record chunks", k, R);
+    } else {
+      choose_orders(&a);
     }
     BatchHeader h;
     std::memset(&h, 0, sizeof h);
@@ -510,8 +511,11 @@ int adha_batched_create(int32_t n_arrays, const adha_remap_desc* descs, int32_t 
   b->smem = (size_t)kWarps * best_region;
   int per_sm = 0;
   auto* k2 = b->direct ? batched_kernel<true> : batched_kernel<false>;
-  e = cudaFuncSetAttribute(k2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b->smem);
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k2, kThreads, b->smem);
+  if (int rc = allow_smem(reinterpret_cast<const void*>(k2), b->smem, "cudaFuncSetAttribute(batched)")) {
+    delete b;
+    return rc;
+  }
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k2, kThreads, b->smem);
   if (e != cudaSuccess) {
     delete b;
     return cuda_fail(e, "batched occupancy");

@@ -57,6 +57,13 @@ int sm_count(int* count) {
   return 0;
 }
 
+int allow_smem(const void* fn, size_t smem, const char* what) {
+  if (smem <= 48 * 1024) return 0;
+  // the most a CTA may have, not `smem`: another thread may be about to launch with more
+  const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
+  return e == cudaSuccess ? 0 : cuda_fail(e, what);
+}
+
 // ------------------------------------------------------------------ layouts
 int group_struct(const int* dtype, const std::vector<int>& fields, std::vector<int>* offsets) {
   int pos = 0, align = 1;
@@ -139,7 +146,7 @@ static bool overlap(const void* a, size_t na, const void* b, size_t nb) {
 }
 
 
-void tanh_coefficients(float p[8], float q[8]) {
+static void tanh_polynomials(float p[8], float q[8]) {
   // P_k = (2k+1) P_{k-1} + a P_{k-2}, Q_k likewise; P_{-1} = 1, P_0 = 1, Q_{-1} = 0, Q_0 = 1; k up to 12.
   int64_t pm[8] = {1}, pc[8] = {1}, qm[8] = {0}, qc[8] = {1};
   for (int k = 1; k <= 12; ++k) {
@@ -157,6 +164,16 @@ void tanh_coefficients(float p[8], float q[8]) {
     p[j] = (float)pc[j];
     q[j] = (float)qc[j];
   }
+}
+
+void tanh_coefficients(float p[8], float q[8]) {
+  struct Both {
+    float p[8], q[8];
+    Both() { tanh_polynomials(p, q); }
+  };
+  static const Both both;
+  std::memcpy(p, both.p, sizeof both.p);
+  std::memcpy(q, both.q, sizeof both.q);
 }
 
 // ------------------------------------------------------------------ launch profiler
@@ -262,12 +279,12 @@ static std::string remap_key(const Layout& S, const Layout& D, int64_t n) {
   return "M" + layout_code(S) + ">" + layout_code(D) + size_class(n);
 }
 
-// Whether the cache holds any remap entry: the key of a pair of layouts, a microsecond or two of text, is
-// built only then.
-static bool any_remap_tuned() {
+// Whether the cache holds any entry of a kind ("S", "M" or "F"): a launch's key, a microsecond or two of
+// text, is built only then.
+static bool any_tuned(const char* kind) {
   std::lock_guard<std::mutex> lk(g_tune_mu);
-  const auto it = g_tune.lower_bound("M");
-  return it != g_tune.end() && it->first[0] == 'M';
+  const auto it = g_tune.lower_bound(kind);
+  return it != g_tune.end() && it->first[0] == kind[0];
 }
 
 std::string tuning_key(const Layout& L, const adha_section* s, int64_t n, bool save) { return section_key(L, s, n, save); }
@@ -362,7 +379,7 @@ static long class_conflict_cost(const RemapArgs& a, int c, int order) {
 static std::mutex g_order_mu;
 static std::map<std::vector<int32_t>, std::vector<int32_t>> g_order_cache;
 
-static void choose_orders(RemapArgs* a) {
+void choose_orders(RemapArgs* a) {
   std::vector<int32_t> key = {a->R, a->n_src, a->n_dst, a->n_moves};
   for (int k = 0; k < a->n_src; ++k) key.push_back(a->src[k].stride);
   for (int k = 0; k < a->n_dst; ++k) key.push_back(a->dst[k].stride);
@@ -456,8 +473,9 @@ static int remap_groups(const Layout& S, const void* const* src_ptrs, const Layo
   return 0;
 }
 
+// arguments_only: neither schedule orders nor a grid.
 static int plan_remap(const Layout& S, const void* const* src_ptrs, const Layout& D, void* const* dst_ptrs, int64_t n,
-                      RemapPlan* plan) {
+                      RemapPlan* plan, bool arguments_only = false) {
   std::memset(&plan->args, 0, sizeof plan->args);
   RemapArgs& a = plan->args;
   std::vector<int> build, need;
@@ -508,7 +526,7 @@ static int plan_remap(const Layout& S, const void* const* src_ptrs, const Layout
   for (int j : need) src_rec += S.stride[j];
   for (int d : build) dst_rec += D.stride[d];
   int tuned_pieces = -1, tuned_R = 0;
-  if ((!t_remap_pieces || !t_tile_override) && any_remap_tuned()) {
+  if ((!t_remap_pieces || !t_tile_override) && any_tuned("M")) {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_tune.find(remap_key(S, D, n));
     if (it != g_tune.end() && it->second.first != kOwnChoice) {
@@ -569,6 +587,7 @@ static int plan_remap(const Layout& S, const void* const* src_ptrs, const Layout
     if (R <= 8) return fail(ADHA_EINVAL, "records too wide for an 8-record chunk (%zu bytes smem)", plan->smem);
     R = std::max(8, R / 2 / 8 * 8);
   }
+  if (arguments_only) return 0;
   choose_orders(&a);
   int blocks = 0;
   if (int rc = cached_occupancy(allow_direct ? 1 : 0, plan->smem, &blocks)) return rc;
@@ -827,7 +846,7 @@ static int plan_section(const Layout& L, void* const* ptrs, const adha_section* 
   SectionArgs& a = plan->args;
   std::memset(&a, 0, sizeof a);
   int tuned_R = t_tile_override, wb_mode = t_writeback_mode, buffers = t_section_buffers;
-  if (!tuned_R && !wb_mode && !buffers) {
+  if (!tuned_R && !wb_mode && !buffers && any_tuned("S")) {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_tune.find(section_key(L, s, n, save != nullptr));
     if (it != g_tune.end() && !(it->second.second & 8)) {   // mode: store mode, + 4 for one chunk buffer per warp
@@ -958,15 +977,16 @@ static int plan_section(const Layout& L, void* const* ptrs, const adha_section* 
 }
 
 int remap_plan_args(const Layout& S, const void* const* src_ptrs, const Layout& D, void* const* dst_ptrs, int64_t n,
-                    int chunk_override, int direct, RemapArgs* out, bool* empty) {
+                    int chunk_override, int direct, bool orders, RemapArgs* out, bool* empty) {
   const int saved = t_tile_override, saved_direct = t_remap_direct;
   t_tile_override = chunk_override;
   t_remap_direct = direct;
   RemapPlan plan;
-  const int rc = plan_remap(S, src_ptrs, D, dst_ptrs, n, &plan);
+  const int rc = plan_remap(S, src_ptrs, D, dst_ptrs, n, &plan, true);
   t_tile_override = saved;
   t_remap_direct = saved_direct;
   if (rc) return rc;
+  if (orders && !plan.empty) choose_orders(&plan.args);
   *out = plan.args;
   *empty = plan.empty;
   return 0;
@@ -996,7 +1016,7 @@ static double section_bytes(const Layout& L, const adha_section* s, int64_t n, b
 // Whether the schedule was tuned to be the faster kernel for this pair of layouts (the key is built only
 // when some remap is tuned).
 static bool remap_tuned(const Layout& S, const Layout& D, int64_t n) {
-  if (!any_remap_tuned()) return false;
+  if (!any_tuned("M")) return false;
   std::lock_guard<std::mutex> lk(g_tune_mu);
   const auto f = g_tune.find(remap_key(S, D, n));
   return f != g_tune.end() && f->second.first != kOwnChoice;
@@ -1118,7 +1138,7 @@ static int plan_fused(const Layout& L, void* const* ptrs, const adha_section* s,
   std::memset(&a, 0, sizeof a);
   int tuned_R = t_tile_override, tuned_buffers = t_fused_buffers;
   bool tuned_jit = false;
-  if (!tuned_R && !tuned_buffers) {
+  if (!tuned_R && !tuned_buffers && any_tuned("F")) {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_tune.find(fused_key(L, s, m, n));
     if (it != g_tune.end()) {   // buffers, + 4 for the run specialised at run time
@@ -1497,7 +1517,7 @@ int run_section_layout(const Layout& L, void* const* ptrs, const adha_section* s
   // tuned (or asked) to run specialised: a one-section run compiled for this section and layout
   if (!save && t_section_jit != 1 && !t_tile_override && !t_writeback_mode && !t_section_buffers) {
     int R = 0, mode = 0;
-    {
+    if (any_tuned("S")) {
       std::lock_guard<std::mutex> lk(g_tune_mu);
       auto it = g_tune.find(section_key(L, s, n, false));
       if (it != g_tune.end()) {

@@ -415,19 +415,17 @@ size_t chain_smem_bytes(const ChainArgs& a, int M, bool backward) {
 
 template <class K>
 static int launch_k(K kernel, const ChainArgs& a, int grid, size_t smem, void* stream) {
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(chain)");
+  if (int rc = allow_smem(reinterpret_cast<const void*>(kernel), smem, "cudaFuncSetAttribute(chain)")) return rc;
   kernel<<<grid, kChainThreads, smem, (cudaStream_t)stream>>>(a);
-  e = cudaGetLastError();
+  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "chain kernel launch");
   return 0;
 }
 
 template <class K>
 static int occ_k(K kernel, size_t smem, int* blocks) {
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(chain)");
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, kernel, kChainThreads, smem);
+  if (int rc = allow_smem(reinterpret_cast<const void*>(kernel), smem, "cudaFuncSetAttribute(chain)")) return rc;
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, kernel, kChainThreads, smem);
   if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor(chain)");
   return 0;
 }

@@ -226,8 +226,8 @@ size_t fused_smem_bytes(const FusedArgs& a) {
 
 template <int M, bool VEC, bool KM>
 static int launch_m(const FusedArgs& a, int grid, size_t smem, void* stream) {
-  cudaError_t e = cudaFuncSetAttribute(fused_kernel<M, VEC, KM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(fused)");
+  if (int rc = allow_smem(reinterpret_cast<const void*>(fused_kernel<M, VEC, KM>), smem, "cudaFuncSetAttribute(fused)")) return rc;
+  cudaError_t e = cudaSuccess;
   if (a.reduce_sec >= 0 && !a.accumulate) {   // the sums are added into a zeroed result
     const SecOp& so = a.sec[a.reduce_sec];
     const int K = so.arg[1], d = so.rd_off[ADHA_F32 + 1] - so.rd_off[ADHA_F32];
@@ -267,9 +267,8 @@ int launch_fused(const FusedArgs& a, int grid, size_t smem, void* stream) {
 
 template <int M, bool VEC, bool KM>
 static int occ_m(size_t smem, int* blocks) {
-  cudaError_t e = cudaFuncSetAttribute(fused_kernel<M, VEC, KM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(fused)");
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, fused_kernel<M, VEC, KM>, kThreads, smem);
+  if (int rc = allow_smem(reinterpret_cast<const void*>(fused_kernel<M, VEC, KM>), smem, "cudaFuncSetAttribute(fused)")) return rc;
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, fused_kernel<M, VEC, KM>, kThreads, smem);
   if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor(fused)");
   return 0;
 }

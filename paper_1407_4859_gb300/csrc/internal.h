@@ -47,6 +47,9 @@ int check_schema(const adha_schema* schema);
 bool same_group(const Layout& a, int ga, const Layout& b, int gb);
 
 int sm_count(int* count);
+// Lets kernel `fn` (without static shared memory) take `smem` bytes of dynamic shared memory; up to 48 KB
+// there is nothing to do, as long as no one sets a lower limit.
+int allow_smem(const void* fn, size_t smem, const char* what);
 
 // ------------------------------------------------------------------ kernel argument blocks
 // (GroupRef, FieldRef, SecOp and FusedArgs are in device_types.h.)
@@ -207,8 +210,10 @@ void fill_secop(const Layout& L, const adha_section* s, SecOp* o);
 void fill_secop_offsets(SecOp* o, const FieldRef* f);
 adha_layout set_layout(const adha_layout_set* s, int l);
 // Remap launch arguments for one array (chunk_override 0 = the default chunk rule).
+// (orders = false: without the schedule orders, which choose_orders adds).
 int remap_plan_args(const Layout& S, const void* const* src_ptrs, const Layout& D, void* const* dst_ptrs, int64_t n,
-                    int chunk_override, int direct, RemapArgs* out, bool* empty);
+                    int chunk_override, int direct, bool orders, RemapArgs* out, bool* empty);
+void choose_orders(RemapArgs* a);
 // Runs fn(ctx) bracketed by the launch profiler's events when profiling is on.
 int profiled_launch(int kind, int op, double bytes, void* stream, int (*fn)(const void*), const void* ctx);
 // Autotuning: the key of a section launch, storing its best shape, thread-local overrides.

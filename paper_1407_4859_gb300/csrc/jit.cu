@@ -19,6 +19,7 @@
 #include <mutex>
 #include <string>
 #include <thread>
+#include <unordered_map>
 #include <vector>
 
 #include "internal.h"
@@ -306,7 +307,26 @@ static int jit_load(const std::string& src, Kernel* out) {
   return 0;
 }
 
-int jit_kernel(const FusedArgs& a, int F, int buffers, bool compile, const void** fn, std::string* why) {
+// Kernels by the run they were made for: the launch arguments without their addresses and record counts,
+// which is all that the source text is made from.  A launch finds its kernel here without writing the
+// text (tens of microseconds of string work).
+static std::mutex g_shape_mu;
+static std::unordered_map<std::string, const void*>* g_shapes = new std::unordered_map<std::string, const void*>();
+
+static std::string shape_of(const FusedArgs& a, int F, int buffers) {
+  FusedArgs k = a;
+  k.n = k.n_chunks = 0;
+  k.perm = nullptr;
+  for (int g = 0; g <= kMaxGroups; ++g) k.load[g].ptr = nullptr;
+  for (int f = 0; f < kMaxFields; ++f) k.f[f].g = nullptr;
+  for (int s = 0; s < a.n_sec; ++s) k.sec[s].aux = nullptr;
+  std::string out(reinterpret_cast<const char*>(&k), offsetof(FusedArgs, sec) + a.n_sec * sizeof(SecOp));
+  const int extra[2] = {F, buffers};
+  out.append(reinterpret_cast<const char*>(extra), sizeof extra);
+  return out;
+}
+
+static int jit_kernel_by_source(const FusedArgs& a, int F, int buffers, bool compile, const void** fn, std::string* why) {
   std::string src;
   if (!jit_source(a, F, buffers, &src, why)) return fail(ADHA_ENOTIMPL, "fused run not specialised: %s", why->c_str());
   if (!compile) {
@@ -322,6 +342,22 @@ int jit_kernel(const FusedArgs& a, int F, int buffers, bool compile, const void*
   Kernel k;
   if (int rc = jit_load(src, &k)) return rc;
   *fn = reinterpret_cast<const void*>(k.fn);
+  return 0;
+}
+
+int jit_kernel(const FusedArgs& a, int F, int buffers, bool compile, const void** fn, std::string* why) {
+  const std::string shape = shape_of(a, F, buffers);
+  {
+    std::lock_guard<std::mutex> lk(g_shape_mu);
+    const auto it = g_shapes->find(shape);
+    if (it != g_shapes->end()) {
+      *fn = it->second;
+      return 0;
+    }
+  }
+  if (int rc = jit_kernel_by_source(a, F, buffers, compile, fn, why)) return rc;
+  std::lock_guard<std::mutex> lk(g_shape_mu);
+  (*g_shapes)[shape] = *fn;
   return 0;
 }
 
@@ -362,9 +398,8 @@ int jit_occupancy(const void* fn, size_t smem, int* blocks) {
         return 0;
       }
   }
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(fused run)");
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, fn, kThreads, smem);
+  if (int rc = allow_smem(fn, smem, "cudaFuncSetAttribute(fused run)")) return rc;
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, fn, kThreads, smem);
   if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor(fused run)");
   std::lock_guard<std::mutex> lk(g_cache_mu);
   for (auto& kv : *g_cache)
@@ -376,8 +411,8 @@ int jit_occupancy(const void* fn, size_t smem, int* blocks) {
 }
 
 int launch_fused_jit(const void* fn, const FusedArgs& a, int grid, size_t smem, void* stream) {
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(fused run)");
+  if (int rc = allow_smem(fn, smem, "cudaFuncSetAttribute(fused run)")) return rc;
+  cudaError_t e = cudaSuccess;
   void* args[] = {const_cast<FusedArgs*>(&a)};
   e = cudaLaunchKernel(fn, dim3(grid), dim3(kThreads), args, smem, (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(e, "specialised fused run launch");

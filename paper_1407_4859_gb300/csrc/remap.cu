@@ -364,10 +364,9 @@ size_t columns_smem_bytes(const ColumnArgs& a) {
 
 template <int M, bool STAGED>
 static int launch_c(const ColumnArgs& a, int grid, size_t smem, void* stream) {
-  cudaError_t e = cudaFuncSetAttribute(column_kernel<M, STAGED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(columns)");
+  if (int rc = allow_smem(reinterpret_cast<const void*>(column_kernel<M, STAGED>), smem, "cudaFuncSetAttribute(columns)")) return rc;
   column_kernel<M, STAGED><<<grid, kThreads, smem, (cudaStream_t)stream>>>(a);
-  e = cudaGetLastError();
+  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "column remap launch");
   return 0;
 }
@@ -382,9 +381,8 @@ int launch_columns(const ColumnArgs& a, int grid, size_t smem, void* stream) {
 
 template <int M, bool STAGED>
 static int occ_c(size_t smem, int* blocks) {
-  cudaError_t e = cudaFuncSetAttribute(column_kernel<M, STAGED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(columns)");
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, column_kernel<M, STAGED>, kThreads, smem);
+  if (int rc = allow_smem(reinterpret_cast<const void*>(column_kernel<M, STAGED>), smem, "cudaFuncSetAttribute(columns)")) return rc;
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, column_kernel<M, STAGED>, kThreads, smem);
   if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor(columns)");
   return 0;
 }
@@ -396,10 +394,9 @@ int columns_occupancy(int R, bool staged, size_t smem, int* blocks) {
 
 template <bool DIRECT>
 static int launch_d(const RemapArgs& a, int grid, size_t smem, void* stream) {
-  cudaError_t e = cudaFuncSetAttribute(remap_kernel<DIRECT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(remap)");
+  if (int rc = allow_smem(reinterpret_cast<const void*>(remap_kernel<DIRECT>), smem, "cudaFuncSetAttribute(remap)")) return rc;
   remap_kernel<DIRECT><<<grid, kThreads, smem, (cudaStream_t)stream>>>(a);
-  e = cudaGetLastError();
+  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "remap kernel launch");
   return 0;
 }
@@ -411,9 +408,8 @@ int launch_remap(const RemapArgs& a, int grid, size_t smem, void* stream) {
 
 template <bool DIRECT>
 static int occ_d(size_t smem, int* blocks) {
-  cudaError_t e = cudaFuncSetAttribute(remap_kernel<DIRECT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(remap)");
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, remap_kernel<DIRECT>, kThreads, smem);
+  if (int rc = allow_smem(reinterpret_cast<const void*>(remap_kernel<DIRECT>), smem, "cudaFuncSetAttribute(remap)")) return rc;
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, remap_kernel<DIRECT>, kThreads, smem);
   if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor(remap)");
   return 0;
 }

@@ -601,27 +601,27 @@ int adha_run_program(const adha_schema* schema, int64_t n, const adha_layout* in
     Arena dry;
     dry.base = static_cast<uint8_t*>(workspace);
     dry.size = workspace ? ws_bytes : 0;
-    Layout c = in;
+    const Layout* c = &in;
     std::vector<void*> cp(in.n_groups, nullptr);
     for (int g = 0; g < in.n_groups; ++g) cp[g] = in_ptrs ? in_ptrs[g] : nullptr;
     for (int k = 0; k < n_sec; k += plan->window_len[k]) {
       const Layout& D = cand[plan->layout_of_section[k]];
-      if (!same_layout(c, D)) {
+      if (c != &D && !same_layout(*c, D)) {
         std::vector<void*> dp(D.n_groups, nullptr);
-        std::vector<bool> kept(c.n_groups, false);
+        std::vector<bool> kept(c->n_groups, false);
         for (int g = 0; g < D.n_groups; ++g) {
-          for (int j = 0; j < c.n_groups; ++j)
-            if (same_group(D, g, c, j)) {
+          for (int j = 0; j < c->n_groups; ++j)
+            if (same_group(D, g, *c, j)) {
               dp[g] = cp[j];
               kept[j] = true;
             }
           if (!dp[g] && !(dp[g] = dry.alloc((size_t)n * D.stride[g])))
             return fail(ADHA_ENOMEM, "program workspace of %zu bytes is too small for the plan", ws_bytes);
         }
-        for (int j = 0; j < c.n_groups; ++j)
+        for (int j = 0; j < c->n_groups; ++j)
           if (!kept[j] && cp[j] && dry.owns(cp[j])) dry.release(cp[j]);
-        c = D;
-        cp = dp;
+        c = &D;
+        cp.swap(dp);
       }
       const int m = plan->window_len[k];
       if (m > 1 && !fusable_run(D, &sections[k], m))
@@ -633,17 +633,17 @@ int adha_run_program(const adha_schema* schema, int64_t n, const adha_layout* in
   Arena arena;
   arena.base = static_cast<uint8_t*>(workspace);
   arena.size = workspace ? ws_bytes : 0;
-  Layout cur = in;
+  const Layout* cur = &in;
   std::vector<void*> cur_p(in_ptrs, in_ptrs + in.n_groups);
   for (int k = 0; k < n_sec; k += plan->window_len[k]) {
     const int l = plan->layout_of_section[k];
     const Layout& D = cand[l];
-    if (!same_layout(cur, D)) {
+    if (cur != &D && !same_layout(*cur, D)) {
       std::vector<void*> dp(D.n_groups, nullptr);
-      std::vector<bool> kept(cur.n_groups, false);
+      std::vector<bool> kept(cur->n_groups, false);
       for (int g = 0; g < D.n_groups; ++g) {
-        for (int j = 0; j < cur.n_groups; ++j)
-          if (same_group(D, g, cur, j)) {
+        for (int j = 0; j < cur->n_groups; ++j)
+          if (same_group(D, g, *cur, j)) {
             dp[g] = cur_p[j];
             kept[j] = true;
           }
@@ -653,38 +653,38 @@ int adha_run_program(const adha_schema* schema, int64_t n, const adha_layout* in
         }
       }
       int launched = 0;
-      if (int rc = remap_layouts(cur, cur_p.data(), D, dp.data(), n, stream, &launched)) return rc;
+      if (int rc = remap_layouts(*cur, cur_p.data(), D, dp.data(), n, stream, &launched)) return rc;
       plan->n_remaps += 1;
       plan->n_launches += launched;
-      for (int j = 0; j < cur.n_groups; ++j)
+      for (int j = 0; j < cur->n_groups; ++j)
         if (!kept[j] && arena.owns(cur_p[j])) arena.release(cur_p[j]);
-      cur = D;
-      cur_p = dp;
+      cur = &D;
+      cur_p.swap(dp);
     }
     const int m = plan->window_len[k];
-    if (int rc = m == 1 ? run_section_layout(cur, cur_p.data(), &sections[k], n, nullptr, stream)
-                        : run_fused_layout(cur, cur_p.data(), &sections[k], m, n, stream))
+    if (int rc = m == 1 ? run_section_layout(*cur, cur_p.data(), &sections[k], n, nullptr, stream)
+                        : run_fused_layout(*cur, cur_p.data(), &sections[k], m, n, stream))
       return rc;
     plan->n_launches += n > 0 ? 1 : 0;
   }
   // also when the last layout equals the input's but its groups lie elsewhere (a plan that left that
   // layout and came back to it): identical groups at other addresses are copied
-  bool home = same_layout(cur, in);
+  bool home = same_layout(*cur, in);
   for (int g = 0; g < in.n_groups && home; ++g) home = cur_p[g] == in_ptrs[g];
   if (back && !home) {
     std::vector<void*> dp(in_ptrs, in_ptrs + in.n_groups);
     int launched = 0;
-    if (int rc = remap_layouts(cur, cur_p.data(), in, dp.data(), n, stream, &launched)) return rc;
+    if (int rc = remap_layouts(*cur, cur_p.data(), in, dp.data(), n, stream, &launched)) return rc;
     plan->n_remaps += 1;
     plan->n_launches += launched;
-    cur = in;
-    cur_p = dp;
+    cur = &in;
+    cur_p.swap(dp);
   }
   plan->final_layout = -1;
   for (int l = 0; l < L && plan->final_layout < 0; ++l)
-    if (same_layout(cur, cand[l])) plan->final_layout = l;
-  plan->final_n_groups = cur.n_groups;
-  for (int g = 0; g < cur.n_groups; ++g) plan->final_ptrs[g] = cur_p[g];
+    if (same_layout(*cur, cand[l])) plan->final_layout = l;
+  plan->final_n_groups = cur->n_groups;
+  for (int g = 0; g < cur->n_groups; ++g) plan->final_ptrs[g] = cur_p[g];
   return 0;
 }
 

@@ -230,8 +230,8 @@ size_t section_smem_bytes(const SectionArgs& a) {
 
 template <int OP, int M, bool VEC>
 static int launch_om(const SectionArgs& a, int grid, size_t smem, void* stream) {
-  cudaError_t e = cudaFuncSetAttribute(section_kernel<OP, M, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(section)");
+  if (int rc = allow_smem(reinterpret_cast<const void*>(section_kernel<OP, M, VEC>), smem, "cudaFuncSetAttribute(section)")) return rc;
+  cudaError_t e = cudaSuccess;
   if (OP == ADHA_OP_REDUCE && !a.accumulate) {   // the sums are added into a zeroed result
     const int K = a.s.arg[1], d = a.s.rd_off[ADHA_F32 + 1] - a.s.rd_off[ADHA_F32];
     e = cudaMemsetAsync(const_cast<void*>(a.s.aux), 0, (size_t)K * (d + 1) * 8, (cudaStream_t)stream);
@@ -258,9 +258,8 @@ static int launch_op(const SectionArgs& a, int grid, size_t smem, void* stream) 
 
 template <int OP, int M, bool VEC>
 static int occ_om(size_t smem, int* blocks) {
-  cudaError_t e = cudaFuncSetAttribute(section_kernel<OP, M, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(section)");
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, section_kernel<OP, M, VEC>, kThreads, smem);
+  if (int rc = allow_smem(reinterpret_cast<const void*>(section_kernel<OP, M, VEC>), smem, "cudaFuncSetAttribute(section)")) return rc;
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, section_kernel<OP, M, VEC>, kThreads, smem);
   if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor(section)");
   return 0;
 }
