@@ -1434,11 +1434,11 @@ static int run_chain(const Layout& L, void* const* ptrs, const void* const* gin,
   tanh_coefficients(tp, tq);
   for (int j = 0; j < 8; ++j) {
     a.tanh_p[j] = pair(tp[j]);
-    a.tanh_q[j] = pair(tq[j]);
+    a.tanh_qn[j] = pair(-tq[j]);
   }
-  // records per lane: the most that leave 12 (forward) or 8 (backward) warps per SM
+  // records per lane: two, fewer where that leaves less than 12 (forward) or 8 (backward) warps per SM
   const int per_warp = 128 * (backward ? 2 * a.n_rows + a.n_tape : a.n_rows), warps = backward ? 8 : 12;
-  int M = 4;
+  int M = 2;
   while (M > 1 && (size_t)warps * M * per_warp > kSmemPerSM - 16 * 1024) M /= 2;
   // few records: short chunks, so that every SM has work
   int sms = 0;
@@ -1449,10 +1449,8 @@ static int run_chain(const Layout& L, void* const* ptrs, const void* const* gin,
   for (int k = 0; k < m; ++k) {
     int x, y, z;
     chain_operands(&s[k], &x, &y, &z);
-    a.sec[k] = ChainSec{s[k].op, row_of[x] * row_bytes, row_of[y] * row_bytes, row_of[z] * row_bytes,
-                        0.0f, 0.0f, tape[k] < 0 ? -1 : tape[k] * row_bytes, 0};
-    a.sec[k].a = s[k].fparam[0];
-    a.sec[k].b = s[k].fparam[1];
+    a.sec[k] = ChainSec{s[k].op, row_of[x] * row_bytes, row_of[y] * row_bytes, row_of[z] * row_bytes, s[k].fparam[0],
+                        s[k].fparam[1], tape[k] < 0 ? -1 : tape[k] * row_bytes, 0};
     if (live[k]) a.live[a.n_live++] = a.sec[k];
   }
   const size_t smem = chain_smem_bytes(a, M, backward);
@@ -1461,7 +1459,7 @@ static int run_chain(const Layout& L, void* const* ptrs, const void* const* gin,
   if (int rc = cached_occupancy(300 + 10 * M + (backward ? 1 : 0), smem, &blocks)) return rc;
   if (blocks < 1) return fail(ADHA_ENOTIMPL, "kernel does not fit on an SM");
   const int64_t want = (a.n_chunks + kChainThreads / 32 - 1) / (kChainThreads / 32);
-  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)sms * blocks, want));
+  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)sms * blocks * (backward ? 1 : 16), want));
   const int n_saved = __builtin_popcountll(written), n_touched = __builtin_popcountll(touched);
   // what the pass has to move: the touched fields in, the written ones out and saved; backward the
   // gradients in and out, the saved values in, and the state back

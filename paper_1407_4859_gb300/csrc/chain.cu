@@ -19,18 +19,19 @@
 // t = tanh(x) from the section's own result).  Only needed versions go to the tape when they are
 // overwritten, and only sections that lead to one are run again.
 //
-// M: as many records per lane as leave 12 warps per SM (forward) or 8 (backward) in the shared
-// memory that the rows and the tape take; the walk's per-section work (operands, branch, loop) is
-// shared by a lane's M records, and below those warp counts its latency shows.  Measured, 64
-// sections (23 of 24 fields written, 39 run again, 14 tape values) over 2^24 records, one array per
-// field:
-//   M        4        2        1
-//   forward  0.97 ms  1.08 ms  2.13 ms   (64 section launches with saves: 2.8 ms)
-//   backward 2.90 ms  2.24 ms  3.39 ms   (64 adjoint launches and a copy of the gradients: 6.1 ms)
-// What bounds it now (ncu): the walk's chains of dependent shared-memory loads and packed
-// arithmetic at 8-16 warps per SM (issue active 54-56%); HBM is at a half (forward) and a third
-// (backward).  Operands from the parameter space instead of shared memory one section ahead:
-// 1.07 and 2.47 ms.
+// M: two records per lane (one packed pair), one where the rows and the tape of two leave fewer than 12
+// warps per SM (forward) or 8 (backward) in shared memory.  The walk's per-section work (operands,
+// branch, loop) is shared by a lane's records, but with four the warps that are left show the walk's
+// latency.  The forward pass gets 16 waves of CTAs, which evens out the SMs' distances from memory;
+// the backward pass is not bound by it.  Measured, 64 sections (23 of 24 fields written, 39 run
+// again, 14 tape values) over 2^24 records, one array per field:
+//   M         4                2                1
+//   forward   0.94 - 0.97 ms   0.91 (one wave: 1.00)   2.1     (64 section launches with saves: 2.8 ms)
+//   backward  3.07 ms          2.06 ms          2.58    (64 adjoint launches and a copy of the gradients: 6.1 ms)
+// What bounds it now: forward HBM at 0.78 of the copy bandwidth; backward the walk's chains of dependent
+// shared-memory loads and packed arithmetic at 12 warps per SM.  Operands from the parameter space
+// instead of shared memory one section ahead: 1.07 and 2.47 ms; two IEEE divisions per tanh pair
+// instead of tanh_pair's quotient: backward 2.24 ms.
 #include <cuda_runtime.h>
 
 #include "internal.h"
@@ -52,20 +53,14 @@ struct LaneVec {
   static constexpr int H = (M + 1) / 2;
   unsigned long long p[H];
   __device__ __forceinline__ void load(const uint8_t* q) {
-    if constexpr (M == 4) {
-      const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(q);
-      p[0] = v.x;
-      p[1] = v.y;
-    } else if constexpr (M == 2) {
+    if constexpr (M == 2) {
       p[0] = *reinterpret_cast<const unsigned long long*>(q);
     } else {
       p[0] = f2_pack(*reinterpret_cast<const float*>(q), 0.0f);
     }
   }
   __device__ __forceinline__ void store(uint8_t* q) const {
-    if constexpr (M == 4) {
-      *reinterpret_cast<ulonglong2*>(q) = make_ulonglong2(p[0], p[1]);
-    } else if constexpr (M == 2) {
+    if constexpr (M == 2) {
       *reinterpret_cast<unsigned long long*>(q) = p[0];
     } else {
       float lo, hi;
@@ -74,29 +69,6 @@ struct LaneVec {
     }
   }
 };
-
-// tanh_cf on both halves: the polynomials packed, the divisions one by one.  A saturated half is
-// evaluated at 0 instead (its quotient is not used), so that no half takes the division's slow path.
-__device__ __forceinline__ unsigned long long tanh_pair(unsigned long long x, const unsigned long long* P,
-                                                        const unsigned long long* Q, unsigned long long nz) {
-  float lo, hi;
-  f2_unpack(x, &lo, &hi);
-  const bool sl = fabsf(lo) >= 9.0f, sh = fabsf(hi) >= 9.0f;
-  const unsigned long long xe = f2_pack(sl ? 0.0f : lo, sh ? 0.0f : hi);
-  const unsigned long long a = f2_mul_alone(xe, xe, nz);
-  unsigned long long q = Q[6], p = P[6];
-#pragma unroll
-  for (int j = 5; j >= 0; --j) {
-    q = f2_add_rn(f2_mul_alone(q, a, nz), Q[j]);
-    p = f2_add_rn(f2_mul_alone(p, a, nz), P[j]);
-  }
-  float nl, nh, dl, dh;
-  f2_unpack(f2_mul_alone(xe, q, nz), &nl, &nh);
-  f2_unpack(p, &dl, &dh);
-  const float tl = sl ? copysignf(1.0f, lo) : __fdiv_rn(nl, dl);
-  const float th = sh ? copysignf(1.0f, hi) : __fdiv_rn(nh, dh);
-  return f2_pack(tl, th);
-}
 
 // One section on the lane's records (`s`: the lane's first record of row 0); TAPE: z's value from
 // before it goes to its tape slot, if it has one.
@@ -336,7 +308,7 @@ __global__ void __launch_bounds__(kChainThreads) chain_forward_kernel(const __gr
     for (int s = 0; s < a.n_sec; ++s) {
       const ChainSec c = next;
       next = sec[min(s + 1, a.n_sec - 1)];
-      chain_section<M, false>(c, mine, nullptr, a.tanh_p, a.tanh_q, a.neg_zero);
+      chain_section<M, false>(c, mine, nullptr, a.tanh_p, a.tanh_qn, a.neg_zero);
     }
     __syncwarp();
     if (whole) store_rows<M, kState, true>(a, rows, S, i0, lane);
@@ -383,7 +355,7 @@ __global__ void __launch_bounds__(kChainThreads) chain_backward_kernel(const __g
     for (int s = 0; s < a.n_live; ++s) {
       const ChainSec c = next;
       next = live[min(s + 1, a.n_live - 1)];
-      chain_section<M, true>(c, S + at, T + at, a.tanh_p, a.tanh_q, a.neg_zero);
+      chain_section<M, true>(c, S + at, T + at, a.tanh_p, a.tanh_qn, a.neg_zero);
     }
     next = sec[a.n_sec - 1];
     cp_async_wait<0>();
@@ -431,21 +403,15 @@ static int occ_k(K kernel, size_t smem, int* blocks) {
 }
 
 int launch_chain(const ChainArgs& a, int M, bool backward, int grid, size_t smem, void* stream) {
-  if (backward) return M == 4   ? launch_k(chain_backward_kernel<4>, a, grid, smem, stream)
-                       : M == 2 ? launch_k(chain_backward_kernel<2>, a, grid, smem, stream)
-                                : launch_k(chain_backward_kernel<1>, a, grid, smem, stream);
-  return M == 4   ? launch_k(chain_forward_kernel<4>, a, grid, smem, stream)
-         : M == 2 ? launch_k(chain_forward_kernel<2>, a, grid, smem, stream)
-                  : launch_k(chain_forward_kernel<1>, a, grid, smem, stream);
+  if (backward) return M == 2 ? launch_k(chain_backward_kernel<2>, a, grid, smem, stream)
+                              : launch_k(chain_backward_kernel<1>, a, grid, smem, stream);
+  return M == 2 ? launch_k(chain_forward_kernel<2>, a, grid, smem, stream)
+                : launch_k(chain_forward_kernel<1>, a, grid, smem, stream);
 }
 
 int chain_occupancy(int M, bool backward, size_t smem, int* blocks) {
-  if (backward) return M == 4   ? occ_k(chain_backward_kernel<4>, smem, blocks)
-                       : M == 2 ? occ_k(chain_backward_kernel<2>, smem, blocks)
-                                : occ_k(chain_backward_kernel<1>, smem, blocks);
-  return M == 4   ? occ_k(chain_forward_kernel<4>, smem, blocks)
-         : M == 2 ? occ_k(chain_forward_kernel<2>, smem, blocks)
-                  : occ_k(chain_forward_kernel<1>, smem, blocks);
+  if (backward) return M == 2 ? occ_k(chain_backward_kernel<2>, smem, blocks) : occ_k(chain_backward_kernel<1>, smem, blocks);
+  return M == 2 ? occ_k(chain_forward_kernel<2>, smem, blocks) : occ_k(chain_forward_kernel<1>, smem, blocks);
 }
 
 }  // namespace adha

@@ -186,7 +186,7 @@ struct ChainArgs {
   float* saved;
   unsigned long long neg_zero;   // the pair (-0, -0) (see f2_mul_alone)
   int32_t n_rows, n_sec, n_live, n_tape, n_wide, n_copy;
-  unsigned long long tanh_p[8], tanh_q[8];   // each coefficient as a pair
+  unsigned long long tanh_p[8], tanh_qn[8];   // the coefficients of P and -Q as pairs
   int8_t wide_row[kMaxFields], wide_len[kMaxFields], wide_written[kMaxFields];   // groups of two or more fields
   ChainRow row[kMaxFields];
   ChainCopy copy[kMaxGroups];

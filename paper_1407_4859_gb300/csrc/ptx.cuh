@@ -63,6 +63,13 @@ __device__ __forceinline__ unsigned long long f2_add_rn(unsigned long long a, un
   return r;
 }
 
+// 1/x within an ulp.
+__device__ __forceinline__ float rcp_approx(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
 // a * b rounded on its own, as fma(a, b, -0): ptxas contracts mul.rn.f32x2 followed by add.rn.f32x2 (or
 // sub) into one fma, whatever -fmad says (measured: equal to fmaf on 4096 of 4096 random pairs,
 // to the separate operations on 3229), so a product that is added to must not be a mul.  neg_zero

@@ -70,3 +70,24 @@ def test_chain_equals_oracle(P, layout, F, used, count, n):
         for j, f in enumerate(g):
             assert np.array_equal(x.grad[:, j].cpu().numpy().view(np.uint32), want[f].view(np.uint32)), "grad %d" % f
             assert np.array_equal(t.detach()[:, j].cpu().numpy().view(np.uint32), fields[f].view(np.uint32)), f
+
+
+def test_tanh_of_every_float(P):
+    """The chain run's tanh (packed, with a quotient of its own) equals the section kernel's (one IEEE
+    division) for all 2^32 floats, NaN for NaN."""
+    n = 1 << 24
+    sec = synth.Section("tanh", (0, 1), frozenset([0]), frozenset([1]))
+    S, aos, soa = P.Schema([0, 0]), P.Layout.aos(2), P.Layout.soa(2)
+    from paper_1407_4859_gb300._lib import adha_section
+    secs = (adha_section * 1)(P.c_section(sec))
+    saved = torch.empty(n, dtype=torch.float32, device="cuda")
+    base = torch.arange(n, dtype=torch.int64, device="cuda")
+    for k in range(256):
+        x = (base + (k << 24)).to(torch.int32).view(torch.float32)
+        both = torch.stack([x, torch.zeros_like(x)], dim=1)
+        P.adha_run_section(S, n, aos, [both], secs[0])
+        z = torch.zeros_like(x)
+        P.adha_chain_forward(S, n, soa, [x, z], secs, saved)
+        want, got = both[:, 1].view(torch.int32), z.view(torch.int32)
+        same = (want == got) | (torch.isnan(both[:, 1]) & torch.isnan(z))
+        assert bool(same.all()), (k, x[~same][:4].tolist(), both[:, 1][~same][:4].tolist(), z[~same][:4].tolist())
