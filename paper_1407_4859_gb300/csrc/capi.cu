@@ -430,10 +430,10 @@ static int cached_occupancy(int kind, size_t smem, int* blocks) {
       return 0;
     }
   }
-  // kinds: < 100 remap (direct or not), 100.. remap by columns (32, 64, 128 records, + 10 unstaged), 200 + 10*M + vec + 2*km fused run, 300 + 10*M + backward chain
+  // kinds: < 100 remap (direct or not), 100.. remap by columns (32, 64, 128 records), 200 + 10*M + vec + 2*km fused run, 300 + 10*M + backward chain
   // run, 1000 + 1000*op + R + vec section
   const int rc = kind < 100     ? remap_occupancy(kind, smem, blocks)
-                 : kind < 150   ? columns_occupancy(32 << (kind - 100) % 10, kind < 110, smem, blocks)
+                 : kind < 150   ? columns_occupancy(32 << (kind - 100), smem, blocks)
                  : kind >= 1000 ? section_occupancy(kind / 1000 - 1, kind % 1000 & ~1, kind & 1, smem, blocks)
                  : kind >= 300 ? chain_occupancy((kind - 300) / 10, (kind - 300) % 10 != 0, smem, blocks)
                               : fused_occupancy((kind - 200) / 10, ((kind - 200) % 10) & 1, ((kind - 200) % 10) >> 1,
@@ -603,39 +603,43 @@ static int plan_columns(const Layout& S, const void* const* src_ptrs, const Layo
   // destination groups carried whole from the input buffer: the same fields, no padding
   int carried[kMaxGroups];   // built group -> source group, -1 otherwise
   int in_rec = 0, out_rec = 0;
-  bool padding = false, narrow = true, any_carried = false;
+  bool padding = false;
   for (int d : build) {
     int data = 0;
     for (int f : D.groups[d]) data += dtype_size(D.dtype[f]);
     carried[d] = -1;
     for (int j : need)
       if (data == D.stride[d] && same_group(D, d, S, j)) carried[d] = j;
-    any_carried = any_carried || carried[d] >= 0;
     if (carried[d] >= 0 || D.groups[d].size() == 1) continue;
     out_rec += staged_stride(D.stride[d]);
     padding = padding || data != D.stride[d];
   }
-  for (int j : need) {
-    in_rec += staged_stride(S.stride[j]);
-    narrow = narrow && S.groups[j].size() == 1 && S.stride[j] >= 4;
+  for (int j : need) in_rec += staged_stride(S.stride[j]);
+  // Records per chunk and waves of CTAs.  One buffer per warp.  A CTA has little to set up, and CTAs handed
+  // out as others finish even out the SMs' different distances from memory (80-byte structs to one
+  // array per field, us per 1 GB moved: 169 with one wave, 160 with 4, 154 with 16), except where
+  // every chunk gathers many slices.  By the schedule -> by columns, us per 1 GB:
+  // * structs to one array per field: 80 bytes 181 -> 154, 24 bytes 175 -> 151, 132 bytes 180 -> 154;
+  // * narrow records (both sides' buffers of 64 or more records leave 16 warps per SM) into several
+  //   structs or back: 36 bytes 171 -> 149, back 172 -> 152, 56 bytes 166 -> 157, back 167 -> 162;
+  // * wide records, 64 records while they leave 8 warps: one array per field into structs, one wave:
+  //   80 bytes 183 -> 158, 96 bytes 185 -> 172, 110 bytes of mixed types 219 -> 181, 132 bytes 183 in
+  //   both; structs into several structs, 8 waves: 92 bytes 249 -> 198, 116 bytes 205 -> 204.
+  const int total = in_rec + out_rec;
+  const bool several = need.size() > 2;
+  bool table = false;   // the sources come in through the piece table
+  int R, waves;
+  if (out_rec == 0) {
+    R = total <= 96 ? 128 : 64;
+    waves = 16;
+  } else if (total <= 112 && need.size() <= 8) {
+    R = total <= 80 ? 128 : 64;
+    waves = need.size() == 1 ? 16 : 8;
+  } else {
+    R = total <= (several ? 220 : 140) ? 64 : 32;
+    waves = several ? 1 : 8;
+    table = several;
   }
-  // Which form, if any (us per 1 GB moved; by the schedule -> by columns):
-  // * every source through the chunk buffer, one buffer per warp, and 8 or 16 times as many CTAs as are
-  //   resident: a CTA has little to set up, and CTAs handed out as others finish even out the SMs'
-  //   different distances from memory (80-byte structs to one array per field: 169 with one wave of
-  //   CTAs, 160 with 4, 154 with 16).  For structs to one array per field 80 bytes 181 -> 154, 24
-  //   bytes 175 -> 151, 132 bytes 180 -> 154; into several structs or back, where the records of both
-  //   sides are narrow enough for 8 warps of 128 records per SM: 36 bytes 171 -> 149, back 172 -> 153,
-  //   56 bytes 166 -> 160, back 167 -> 163.  Staging many slices of few bytes costs more than it
-  //   saves (12 one-field sources into 52-byte structs: 233 -> 244), wider records leave too few warps
-  //   (116 bytes into eight structs: 205 -> 240).
-  // * sources of one field, 4 or 8 bytes, read straight from their arrays into structs (80 bytes: 183 ->
-  //   158, 96 bytes 185 -> 172; one wave: 163 and 184 with 16).
-  // * neither (wide records between several structs, 2-byte fields into wide structs): by the schedule.
-  const bool staged = out_rec == 0 || (in_rec + out_rec <= 112 && need.size() <= 8);
-  if (!staged && (!narrow || any_carried)) return 0;
-  if (!staged) in_rec = 0;
-  int R = staged && in_rec + out_rec <= (out_rec ? 112 : 96) ? 128 : 64;
   const int nb = 1;
   auto warp_bytes = [&](int r) { return r * (nb * in_rec + out_rec); };
   int sms = 0;
@@ -653,7 +657,6 @@ static int plan_columns(const Layout& S, const void* const* src_ptrs, const Layo
   int in_at[kMaxGroups], off = 0;
   for (int j : need) {
     in_at[j] = off;
-    if (!staged) continue;
     ColSlice& q = a.in[a.n_in++];
     q.ptr = static_cast<const uint8_t*>(src_ptrs[j]);
     q.at = (uint16_t)off;
@@ -681,8 +684,7 @@ static int plan_columns(const Layout& S, const void* const* src_ptrs, const Layo
       const uint16_t so = (uint16_t)(in_at[j] + S.offset_of[f]), ss = (uint16_t)staged_stride(S.stride[j]);
       const uint16_t at = (uint16_t)(off + D.offset_of[f]);
       if (one) moves.push_back({c, {static_cast<const uint8_t*>(dst_ptrs[d]), so, ss, 0, 0}});
-      else if (!staged) moves.push_back({3 + c, {static_cast<const uint8_t*>(src_ptrs[j]), at, (uint16_t)ds, 0, 0}});
-      else moves.push_back({5 + c, {nullptr, so, ss, at, (uint16_t)ds}});
+      else moves.push_back({3 + c, {nullptr, so, ss, at, (uint16_t)ds}});
     }
     if (!one) off += R * ds;
   }
@@ -694,12 +696,17 @@ static int plan_columns(const Layout& S, const void* const* src_ptrs, const Layo
         a.col[k++] = m.m;
         a.cnt[c]++;
       }
+  // Slices of 32 or 64 records are a few pieces each, fewer than a warp has lanes (16 arrays into 80-byte
+  // structs slice by slice: 204); few slices of narrow records are as well copied one by one (30-byte
+  // records 186, by the table 194).
+  if (table)
+    for (int j : need) a.n_pieces += R * S.stride[j] / 16;
   plan->smem = columns_smem_bytes(a);
   if (plan->smem > (size_t)kSmemLimit) return 0;
   int blocks = 0;
-  if (int rc = cached_occupancy((staged ? 100 : 110) + (R == 128 ? 2 : R == 64 ? 1 : 0), plan->smem, &blocks)) return rc;
+  if (int rc = cached_occupancy(100 + (R == 128 ? 2 : R == 64 ? 1 : 0), plan->smem, &blocks)) return rc;
   *fits = true;
-  return finish_grid(a.n_chunks, blocks * (!staged ? 1 : out_rec ? 8 : 16), &plan->grid);
+  return finish_grid(a.n_chunks, blocks * waves, &plan->grid);
 }
 
 // ------------------------------------------------------------------ section planning

@@ -87,10 +87,9 @@ struct RemapArgs {
   Move move[kMaxMoves];
 };
 
-// Remap by columns (remap.cu): lane = record, one step per field.  A destination group of one field is
-// stored straight to global memory (kind A), a source group of one field is read straight from it
-// (kind B) or staged like the wider ones, whose records pass through slices of a chunk buffer (kind C:
-// from an input slice to an output slice).
+// Remap by columns (remap.cu): lane = record, one step per field.  Source groups pass through slices of
+// the input chunk buffer; a destination group of one field is stored straight to global memory (kind
+// A), wider ones are built in the output chunk buffer (kind C).
 struct ColSlice {
   const uint8_t* ptr;   // group buffer
   uint16_t at;          // offset in the warp's input or output chunk buffer
@@ -101,11 +100,11 @@ constexpr uint16_t kColStride = 0x1FFF;
 constexpr uint16_t kColRoom = 1u << 15;     // 16 bytes of room after each staged record (see staged_room)
 constexpr uint16_t kColFromIn = 1u << 14;   // output: the group as it is in the input buffer (same fields, no padding)
 struct ColMove {
-  const uint8_t* g;        // A: the destination array, B: the source array
-  uint16_t off, stride;    // the field in record 0 of the input (A, C) or output (B) buffer, bytes between records
+  const uint8_t* g;        // A: the destination array
+  uint16_t off, stride;    // the field in record 0 of the input buffer, bytes between records
   uint16_t off2, stride2;  // C: the same in the output buffer
 };
-constexpr int kColClasses = 8;   // A of 8, 4, 2 bytes; B of 8, 4; C of 8, 4, 2 (in that order in `col`)
+constexpr int kColClasses = 6;   // A of 8, 4, 2 bytes, then C of 8, 4, 2 (in that order in `col`)
 struct ColumnArgs {
   int64_t n, n_chunks;     // records; whole chunks of R records
   int32_t R;               // 32, 64 or 128; 8 or 16 for wide records
@@ -113,6 +112,7 @@ struct ColumnArgs {
   int32_t in_bytes, out_bytes;
   int32_t buffers;         // chunk buffers per warp: 2 (the next chunk copied in during this one) or 1
   int32_t fill;            // 1: destination structs have padding (zeroed once, never written)
+  int32_t n_pieces;        // > 0: the input's 16-byte pieces through a table of that many (staging.cuh)
   int32_t cnt[kColClasses];
   ColSlice in[kMaxGroups], out[kMaxGroups];
   ColMove col[kMaxFields];
@@ -248,7 +248,7 @@ void tanh_coefficients(float p[8], float q[8]);
 int launch_remap(const RemapArgs& a, int grid, size_t smem, void* stream);
 size_t remap_smem_bytes(const RemapArgs& a);
 int launch_columns(const ColumnArgs& a, int grid, size_t smem, void* stream);
-int columns_occupancy(int R, bool staged, size_t smem, int* blocks);
+int columns_occupancy(int R, size_t smem, int* blocks);
 size_t columns_smem_bytes(const ColumnArgs& a);
 int launch_section(const SectionArgs& a, int grid, size_t smem, void* stream);
 size_t section_smem_bytes(const SectionArgs& a);

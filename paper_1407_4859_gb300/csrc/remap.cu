@@ -26,6 +26,7 @@
 #include "internal.h"
 #include "ptx.cuh"
 #include "remap_common.cuh"
+#include "staging.cuh"
 
 namespace adha {
 
@@ -126,21 +127,24 @@ size_t remap_smem_bytes(const RemapArgs& a) {
 // Remap by columns: the default for a pair of layouts that has not been tuned.
 //
 // The kernel above moves a chunk element by element through a schedule (three shared-memory
-// accesses and the unpacking per element, a table of R x fields entries built by every CTA, one
-// buffer for each side).  Here a lane is a record and a step is one field of 32 records, so that a
-// field's place is one table entry for the whole chunk and the consecutive records of a one-field
-// group are one coalesced access: such groups need no buffer and no 16-byte copy loop at all.
-//   source struct -> one-field group:  shared load, global store
-//   one-field group -> destination struct:  global load, shared store (cp.async of 4 bytes into place:
-//     190 us where this takes 165; slices of the chunk staged first: 204)
-//   struct -> struct:  shared load, shared store
-// Structs move in and out in 16-byte pieces as above.  Structs of an even number of pieces are staged
-// with 16 bytes of room, or 32 records' fields would lie on a few banks.
-template <int M, bool STAGED>
+// accesses and the unpacking per element, a table of R x fields entries built by every CTA).  Here a
+// lane is a record and a step is one field of 32 records, so that a field's place is one table entry
+// for the whole chunk and the consecutive records of a one-field destination group are one coalesced
+// store: such groups need no output buffer and no 16-byte copy loop.
+//   into a one-field group:  shared load, global store
+//   into a struct:           shared load, shared store; the structs go out in 16-byte pieces
+// Sources come in in 16-byte pieces, slice by slice, or through the piece table of staging.cuh where
+// there are several slices.  Structs of an even number of pieces are staged with 16 bytes of room, or
+// 32 records' fields would lie on a few banks.  (One-field sources read straight into the structs, by
+// 4-byte cp.async or through registers: 190 and 157-184 us per 1 GB where the staged form takes
+// 157-183.)
+template <int M>
 struct Columns {
   const ColumnArgs& a;
   const ColMove* col;
   const ColSlice *in, *out;
+  const StagePiece* tab;   // the input pieces of a chunk, NULL: slice by slice
+  int n_pieces;
   int R, lane;
   uint8_t *ibuf, *obuf;   // the warp's input buffers and its output buffer
 
@@ -160,6 +164,7 @@ struct Columns {
   // The chunk's source slices into buffer b.
   template <bool WHOLE>
   __device__ __forceinline__ void stage(int64_t ch, int b, int cnt) const {
+    if (WHOLE && tab) return stage_chunk(tab, n_pieces, ch, ib(b), lane);
     const uint32_t si = smem_addr(ib(b));
     for (int k = 0; k < a.n_in; ++k) {
       const ColSlice s = in[k];
@@ -191,35 +196,6 @@ struct Columns {
     }
   }
 
-  // B columns at a time, so that B * M loads are in flight before the first store.
-  template <class V, bool WHOLE, int B>
-  __device__ __forceinline__ void columns_in(int k, int64_t i0, int cnt) const {
-    const int64_t at = i0 + lane;
-    V v[B][M];
-#pragma unroll
-    for (int b = 0; b < B; ++b) {
-      const V* src = reinterpret_cast<const V*>(col[k + b].g) + at;
-#pragma unroll
-      for (int m = 0; m < M; ++m)
-        if ((WHOLE && M > 1) || on(m, cnt)) v[b][m] = __ldg(src + m * 32);
-    }
-#pragma unroll
-    for (int b = 0; b < B; ++b) {
-      const ColMove t = col[k + b];
-      uint8_t* dst = obuf + t.off + lane * t.stride;
-#pragma unroll
-      for (int m = 0; m < M; ++m)
-        if ((WHOLE && M > 1) || on(m, cnt)) *reinterpret_cast<V*>(dst + m * 32 * t.stride) = v[b][m];
-    }
-  }
-  template <class V, bool WHOLE>
-  __device__ __forceinline__ void column_in(int k, int end, int64_t i0, int cnt) const {
-    for (; k + 8 <= end; k += 8) columns_in<V, WHOLE, 8>(k, i0, cnt);
-    if (k + 4 <= end) columns_in<V, WHOLE, 4>(k, i0, cnt), k += 4;
-    if (k + 2 <= end) columns_in<V, WHOLE, 2>(k, i0, cnt), k += 2;
-    if (k < end) columns_in<V, WHOLE, 1>(k, i0, cnt);
-  }
-
   template <class V, bool WHOLE>
   __device__ __forceinline__ void column_across(int k, int end, const uint8_t* __restrict__ src0, uint8_t* __restrict__ dst0,
                                                 int cnt) const {
@@ -242,28 +218,17 @@ struct Columns {
   __device__ __forceinline__ void moves(int64_t ch, int b, int cnt) const {
     const int64_t i0 = ch * R;
     const uint8_t* src = ib(b);
-    int k = 0, e = 0;
-    if constexpr (STAGED) {
-      e = a.cnt[0];
-      column_out<unsigned long long, WHOLE>(k, e, src, i0, cnt);
-      k = e, e += a.cnt[1];
-      column_out<uint32_t, WHOLE>(k, e, src, i0, cnt);
-      k = e, e += a.cnt[2];
-      column_out<uint16_t, WHOLE>(k, e, src, i0, cnt);
-    }
-    if constexpr (!STAGED) {
-      k = e, e += a.cnt[3];
-      column_in<unsigned long long, WHOLE>(k, e, i0, cnt);
-      k = e, e += a.cnt[4];
-      column_in<uint32_t, WHOLE>(k, e, i0, cnt);
-      return;
-    }
-    e += a.cnt[3] + a.cnt[4];
-    k = e, e += a.cnt[5];
+    int k = 0, e = a.cnt[0];
+    column_out<unsigned long long, WHOLE>(k, e, src, i0, cnt);
+    k = e, e += a.cnt[1];
+    column_out<uint32_t, WHOLE>(k, e, src, i0, cnt);
+    k = e, e += a.cnt[2];
+    column_out<uint16_t, WHOLE>(k, e, src, i0, cnt);
+    k = e, e += a.cnt[3];
     column_across<unsigned long long, WHOLE>(k, e, src, obuf, cnt);
-    k = e, e += a.cnt[6];
+    k = e, e += a.cnt[4];
     column_across<uint32_t, WHOLE>(k, e, src, obuf, cnt);
-    k = e, e += a.cnt[7];
+    k = e, e += a.cnt[5];
     column_across<uint16_t, WHOLE>(k, e, src, obuf, cnt);
   }
 
@@ -287,8 +252,7 @@ struct Columns {
   }
 };
 
-// STAGED: sources through the chunk buffer (kinds A and C); else straight from their arrays (kind B).
-template <int M, bool STAGED>
+template <int M>
 __global__ void __launch_bounds__(kThreads, 4) column_kernel(const __grid_constant__ ColumnArgs a) {
   extern __shared__ __align__(16) uint8_t smem[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -301,13 +265,21 @@ __global__ void __launch_bounds__(kThreads, 4) column_kernel(const __grid_consta
   for (int k = tid; k < n_col; k += kThreads) col[k] = a.col[k];
   for (int k = tid; k < a.n_in; k += kThreads) in[k] = a.in[k];
   for (int k = tid; k < a.n_out; k += kThreads) out[k] = a.out[k];
-  uint8_t* mine = reinterpret_cast<uint8_t*>(out + a.n_out) + (size_t)warp * (nb * a.in_bytes + a.out_bytes);
+  const int R = M == 1 ? a.R : 32 * M;
+  StagePiece* tab = reinterpret_cast<StagePiece*>(out + a.n_out);
+  for (int q = tid; q < a.n_pieces; q += kThreads) {
+    int p = q * 16, k = 0;
+    while (p >= R * (a.in[k].stride & kColStride)) p -= R * (a.in[k++].stride & kColStride);
+    const int stride = a.in[k].stride & kColStride;
+    const int room = a.in[k].stride & kColRoom ? 16 * (int)__umulhi((unsigned)p, a.in[k].magic) : 0;
+    tab[q] = StagePiece{a.in[k].ptr + p, R * stride, a.in[k].at + p + room};
+  }
+  uint8_t* mine = reinterpret_cast<uint8_t*>(tab + a.n_pieces) + (size_t)warp * (nb * a.in_bytes + a.out_bytes);
   if (a.fill)
     for (int p = lane * 16; p < a.out_bytes; p += 512)
       *reinterpret_cast<uint4*>(mine + nb * a.in_bytes + p) = make_uint4(0, 0, 0, 0);
   __syncthreads();
-  const int R = M == 1 ? a.R : 32 * M;
-  const Columns<M, STAGED> w{a, col, in, out, R, lane, mine, mine + nb * a.in_bytes};
+  const Columns<M> w{a, col, in, out, a.n_pieces ? tab : nullptr, a.n_pieces, R, lane, mine, mine + nb * a.in_bytes};
   const int64_t W = (int64_t)gridDim.x * kWarps;
   // one input buffer: the next chunk may come in once the moves have read this one, unless groups are
   // written from it
@@ -359,37 +331,34 @@ __global__ void __launch_bounds__(kThreads, 4) column_kernel(const __grid_consta
 size_t columns_smem_bytes(const ColumnArgs& a) {
   int n_col = 0;
   for (int k = 0; k < kColClasses; ++k) n_col += a.cnt[k];
-  return (size_t)(n_col + a.n_in + a.n_out) * 16 + (size_t)kWarps * ((size_t)a.buffers * a.in_bytes + a.out_bytes);
+  return (size_t)(n_col + a.n_in + a.n_out + a.n_pieces) * 16 + (size_t)kWarps * ((size_t)a.buffers * a.in_bytes + a.out_bytes);
 }
 
-template <int M, bool STAGED>
+template <int M>
 static int launch_c(const ColumnArgs& a, int grid, size_t smem, void* stream) {
-  if (int rc = allow_smem(reinterpret_cast<const void*>(column_kernel<M, STAGED>), smem, "cudaFuncSetAttribute(columns)")) return rc;
-  column_kernel<M, STAGED><<<grid, kThreads, smem, (cudaStream_t)stream>>>(a);
-  cudaError_t e = cudaGetLastError();
+  if (int rc = allow_smem(reinterpret_cast<const void*>(column_kernel<M>), smem, "cudaFuncSetAttribute(columns)")) return rc;
+  column_kernel<M><<<grid, kThreads, smem, (cudaStream_t)stream>>>(a);
+  const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "column remap launch");
   return 0;
 }
 
 int launch_columns(const ColumnArgs& a, int grid, size_t smem, void* stream) {
-  if (a.cnt[3] + a.cnt[4] > 0)
-    return a.R == 64 ? launch_c<2, false>(a, grid, smem, stream) : launch_c<1, false>(a, grid, smem, stream);
-  return a.R == 128  ? launch_c<4, true>(a, grid, smem, stream)
-         : a.R == 64 ? launch_c<2, true>(a, grid, smem, stream)
-                     : launch_c<1, true>(a, grid, smem, stream);
+  return a.R == 128  ? launch_c<4>(a, grid, smem, stream)
+         : a.R == 64 ? launch_c<2>(a, grid, smem, stream)
+                     : launch_c<1>(a, grid, smem, stream);
 }
 
-template <int M, bool STAGED>
+template <int M>
 static int occ_c(size_t smem, int* blocks) {
-  if (int rc = allow_smem(reinterpret_cast<const void*>(column_kernel<M, STAGED>), smem, "cudaFuncSetAttribute(columns)")) return rc;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, column_kernel<M, STAGED>, kThreads, smem);
+  if (int rc = allow_smem(reinterpret_cast<const void*>(column_kernel<M>), smem, "cudaFuncSetAttribute(columns)")) return rc;
+  const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, column_kernel<M>, kThreads, smem);
   if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor(columns)");
   return 0;
 }
 
-int columns_occupancy(int R, bool staged, size_t smem, int* blocks) {
-  if (!staged) return R == 64 ? occ_c<2, false>(smem, blocks) : occ_c<1, false>(smem, blocks);
-  return R == 128 ? occ_c<4, true>(smem, blocks) : R == 64 ? occ_c<2, true>(smem, blocks) : occ_c<1, true>(smem, blocks);
+int columns_occupancy(int R, size_t smem, int* blocks) {
+  return R == 128 ? occ_c<4>(smem, blocks) : R == 64 ? occ_c<2>(smem, blocks) : occ_c<1>(smem, blocks);
 }
 
 template <bool DIRECT>
