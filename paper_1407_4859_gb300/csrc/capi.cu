@@ -1325,13 +1325,20 @@ static void chain_operands(const adha_section* s, int* x, int* y, int* z) {
   *z = s->op == ADHA_OP_MUL ? s->arg[2] : s->arg[1];
 }
 
-// What the reverse walk needs of each field's versions (version f < F: the field's value before the
-// run; F + k: what section k writes).  adj: read by a mul (its adjoint multiplies by the operands)
-// or made by a tanh (its adjoint takes the result).  live: adj, or an operand on the way to one.
-// The backward pass runs only the live sections again; each puts the value it overwrites on the
-// tape if that value is adj.  tape[k] = slot or -1.  Returns the number of slots.
-static int chain_tape(int F, const adha_section* s, int m, std::vector<int>* tape, std::vector<bool>* live_sec) {
-  std::vector<int> cur(F), vx(m), vy(m);
+// Where the backward pass keeps the values that it needs.  A version of a field is its value before
+// the run (f < F) or what section k writes (F + k).  adj: read by a mul (its adjoint multiplies by the
+// operands) or made by a tanh (its adjoint takes the result): kept to the end.  live: adj, or an
+// operand on the way to one; only the sections that make live versions run again.  Slots F and up
+// hold what does not fit into the fields' own slots; a slot whose version nothing reads any more
+// takes the next one, so that no value is copied.
+struct ChainSlots {
+  std::vector<int> x, y, z;   // per section, slots: what it reads, and (live sections) what it writes
+  std::vector<bool> live;
+  int extra = 0;              // slots beyond the fields' own
+};
+// rows: the fields that have a slot of their own.
+static ChainSlots chain_slots(int F, uint64_t rows, const adha_section* s, int m) {
+  std::vector<int> cur(F), vx(m), vy(m), last(F + m, -1), at(F + m, -1);
   std::vector<bool> adj(F + m, false);
   for (int f = 0; f < F; ++f) cur[f] = f;
   for (int k = 0; k < m; ++k) {
@@ -1345,30 +1352,40 @@ static int chain_tape(int F, const adha_section* s, int m, std::vector<int>* tap
   }
   std::vector<bool> live = adj;
   for (int k = m - 1; k >= 0; --k)
-    if (live[F + k]) live[vx[k]] = live[vy[k]] = true;
-  for (int f = 0; f < F; ++f) cur[f] = f;
-  tape->assign(m, -1);
-  live_sec->assign(m, false);
-  int slots = 0;
-  for (int k = 0; k < m; ++k) {
-    if (!live[F + k]) continue;
-    int x, y, z;
-    chain_operands(&s[k], &x, &y, &z);
-    (*live_sec)[k] = true;
-    if (adj[cur[z]]) (*tape)[k] = slots++;
-    cur[z] = F + k;
+    if (live[F + k])
+      for (int v : {vx[k], vy[k]}) {
+        live[v] = true;
+        last[v] = std::max(last[v], k);
+      }
+  ChainSlots r;
+  std::vector<int> free;
+  for (int f = F - 1; f >= 0; --f) {
+    if (!has(rows, f)) continue;
+    at[f] = f;
+    if (!live[f]) free.push_back(f);
   }
-  return slots;
-}
-
-// Leading sections of s[0..m) that fit one run: at most kMaxChain, and a tape of at most
-// kMaxChainTape values (with the rows of 64 fields and their gradients, eight warps per SM).
-static int chain_window(int F, const adha_section* s, int m) {
-  std::vector<int> tape;
-  std::vector<bool> live;
-  int k = std::min(m, kMaxChain);
-  while (k > 1 && chain_tape(F, s, k, &tape, &live) > kMaxChainTape) k = std::max(1, k - 8);
-  return k;
+  r.x.assign(m, 0);
+  r.y.assign(m, 0);
+  r.z.assign(m, 0);
+  r.live.assign(m, false);
+  for (int k = 0; k < m; ++k) {
+    if (live[F + k]) {
+      // a section reads its operands before it writes: its output may take the slot of one
+      for (int v : {vx[k], vy[k]})
+        if (!adj[v] && last[v] == k) {
+          free.push_back(at[v]);
+          last[v] = -1;   // once, where both operands are the same
+        }
+      if (free.empty()) free.push_back(F + r.extra++);
+      at[F + k] = free.back();
+      free.pop_back();
+      r.live[k] = true;
+    }
+    r.x[k] = at[vx[k]];
+    r.y[k] = at[vy[k]];
+    r.z[k] = at[F + k];
+  }
+  return r;
 }
 
 static uint64_t chain_written(const adha_section* s, int m) {
@@ -1381,6 +1398,24 @@ static uint64_t chain_written(const adha_section* s, int m) {
   return w;
 }
 
+static uint64_t chain_read(const adha_section* s, int m) {
+  uint64_t r = 0;
+  for (int k = 0; k < m; ++k) {
+    int x, y, z;
+    chain_operands(&s[k], &x, &y, &z);
+    r |= 1ull << x | 1ull << y;
+  }
+  return r;
+}
+
+// Leading sections of s[0..m) that fit one run: at most kMaxChain, and at most kMaxChainTape slots
+// beyond the fields' own (with the rows of 64 fields and their gradients, eight warps per SM).
+static int chain_window(int F, const adha_section* s, int m) {
+  int k = std::min(m, kMaxChain);
+  while (k > 1 && chain_slots(F, chain_written(s, k) | chain_read(s, k), s, k).extra > kMaxChainTape) k = std::max(1, k - 8);
+  return k;
+}
+
 static int64_t chain_pitch(int64_t n) { return (n + 127) / 128 * 128; }
 
 // gin, gout: NULL for the forward run.
@@ -1389,16 +1424,8 @@ static int run_chain(const Layout& L, void* const* ptrs, const void* const* gin,
   const bool backward = gin != nullptr;
   ChainArgs a;
   std::memset(&a, 0, sizeof a);
-  std::vector<int> tape;
-  std::vector<bool> live;
-  a.n_tape = chain_tape(L.F, s, m, &tape, &live);
-  const uint64_t written = chain_written(s, m);
-  uint64_t touched = written;
-  for (int k = 0; k < m; ++k) {
-    int x, y, z;
-    chain_operands(&s[k], &x, &y, &z);
-    touched |= 1ull << x | 1ull << y;
-  }
+  const uint64_t written = chain_written(s, m), touched = written | chain_read(s, m);
+  uint64_t rows = 0;
   int row_of[kMaxFields];
   for (int g = 0; g < L.n_groups; ++g) {
     const auto& fields = L.groups[g];
@@ -1425,6 +1452,7 @@ static int run_chain(const Layout& L, void* const* ptrs, const void* const* gin,
       r.stride = L.stride[g];
       r.saved = has(written, f) ? __builtin_popcountll(written & ((1ull << f) - 1)) : -1;
       row_of[f] = a.n_rows++;
+      rows |= 1ull << f;
     }
   }
   a.n = n;
@@ -1443,8 +1471,11 @@ static int run_chain(const Layout& L, void* const* ptrs, const void* const* gin,
     a.tanh_p[j] = pair(tp[j]);
     a.tanh_qn[j] = pair(-tq[j]);
   }
+  ChainSlots slots;
+  if (backward) slots = chain_slots(L.F, rows, s, m);
+  a.n_tape = slots.extra;
   // records per lane: two, fewer where that leaves less than 12 (forward) or 8 (backward) warps per SM
-  const int per_warp = 128 * (backward ? 2 * a.n_rows + a.n_tape : a.n_rows), warps = backward ? 8 : 12;
+  const int per_warp = 128 * (backward ? 2 * a.n_rows + a.n_tape + 1 : a.n_rows), warps = backward ? 8 : 12;
   int M = 2;
   while (M > 1 && (size_t)warps * M * per_warp > kSmemPerSM - 16 * 1024) M /= 2;
   // few records: short chunks, so that every SM has work
@@ -1453,20 +1484,66 @@ static int run_chain(const Layout& L, void* const* ptrs, const void* const* gin,
   while (M > 1 && n < (int64_t)sms * warps * 32 * M) M /= 2;
   a.n_chunks = (n + 32 * M - 1) / (32 * M);
   const int row_bytes = 128 * M;
-  for (int k = 0; k < m; ++k) {
-    int x, y, z;
-    chain_operands(&s[k], &x, &y, &z);
-    a.sec[k] = ChainSec{s[k].op, row_of[x] * row_bytes, row_of[y] * row_bytes, row_of[z] * row_bytes, s[k].fparam[0],
-                        s[k].fparam[1], tape[k] < 0 ? -1 : tape[k] * row_bytes, 0};
-    if (live[k]) a.live[a.n_live++] = a.sec[k];
+  for (int k = 0; k < a.n_rows; ++k) {
+    const ChainRow& r = a.row[k];
+    auto add = [&](int l, const void* p) {
+      a.span[l][a.n_span[l]++] = ChainSpan{const_cast<uint8_t*>(static_cast<const uint8_t*>(p)), k * row_bytes, 0};
+    };
+    const bool array = r.stride == 4;
+    const float* sv = r.saved >= 0 ? saved + r.saved * a.pitch : nullptr;
+    if (!backward) {
+      if (array) add(0, r.state);
+      if (sv) add(1, sv);
+      if (array && sv) add(2, r.state);
+    } else {
+      if (sv) add(0, sv);
+      else if (array) add(0, r.state);
+      if (array && sv) add(1, r.state);
+      if (array) add(2, r.gin), add(3, r.gout);
+    }
+  }
+  if (backward) {
+    auto slot = [&](int v) { return (v < L.F ? row_of[v] : a.n_rows + v - L.F) * row_bytes; };
+    for (int k = 0; k < m; ++k)
+      if (slots.live[k])
+        a.sec[a.n_live++] = ChainSec{s[k].op, slot(slots.x[k]), slot(slots.y[k]), slot(slots.z[k]), s[k].fparam[0], s[k].fparam[1], {}};
+    // the reverse walk; a gradient is zero from where it has been passed on to where it is next added to
+    for (int k = m - 1; k >= 0; --k) {
+      int x, y, z;
+      chain_operands(&s[k], &x, &y, &z);
+      ChainAdj& t = a.adj[m - 1 - k];
+      auto from = [&](int f) { return (has(a.zero_rows, row_of[f]) ? a.n_rows : row_of[f]) * row_bytes; };
+      t.op = s[k].op;
+      t.gz = from(z);
+      a.zero_rows |= 1ull << row_of[z];
+      t.gx_in = from(x);
+      t.gx = row_of[x] * row_bytes;
+      a.zero_rows &= ~(1ull << row_of[x]);
+      if (s[k].op == ADHA_OP_MUL) {
+        t.gy_in = from(y);
+        t.gy = row_of[y] * row_bytes;
+        a.zero_rows &= ~(1ull << row_of[y]);
+        t.vx = slot(slots.x[k]);
+        t.vy = slot(slots.y[k]);
+      } else if (s[k].op == ADHA_OP_TANH) {
+        t.vx = slot(slots.z[k]);
+      } else {
+        t.a = s[k].fparam[0];
+      }
+    }
+  } else {
+    for (int k = 0; k < m; ++k) {
+      int x, y, z;
+      chain_operands(&s[k], &x, &y, &z);
+      a.sec[k] = ChainSec{s[k].op, row_of[x] * row_bytes, row_of[y] * row_bytes, row_of[z] * row_bytes, s[k].fparam[0], s[k].fparam[1], {}};
+    }
   }
   const size_t smem = chain_smem_bytes(a, M, backward);
   if (smem > (size_t)kSmemLimit) return fail(ADHA_EINVAL, "the chain run's records are too wide for a 32-record chunk");
   int blocks = 0;
   if (int rc = cached_occupancy(300 + 10 * M + (backward ? 1 : 0), smem, &blocks)) return rc;
   if (blocks < 1) return fail(ADHA_ENOTIMPL, "kernel does not fit on an SM");
-  const int64_t want = (a.n_chunks + kChainThreads / 32 - 1) / (kChainThreads / 32);
-  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)sms * blocks * (backward ? 1 : 16), want));
+  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)sms * blocks * 16, a.n_chunks));
   const int n_saved = __builtin_popcountll(written), n_touched = __builtin_popcountll(touched);
   // what the pass has to move: the touched fields in, the written ones out and saved; backward the
   // gradients in and out, the saved values in, and the state back

@@ -14,24 +14,31 @@
 // arithmetic (the tanh polynomials), not memory: a lane's records are carried as pairs in the packed
 // fp32 instructions (each half an IEEE operation on its own, as in the per-record rule).
 //
-// What the reverse walk needs of the values in between is found on the host (chain.cu's planner): a
+// What the reverse walk needs of the values in between is found on the host (chain_slots in capi.cu): a
 // version of a field is needed if a mul reads it or a tanh made it (the tanh adjoint takes
-// t = tanh(x) from the section's own result).  Only needed versions go to the tape when they are
-// overwritten, and only sections that lead to one are run again.
+// t = tanh(x) from the section's own result).  Only sections that lead to a needed version are run
+// again, and each version gets a slot of its own, so that nothing is copied or restored: the slot of a
+// version that is no longer needed, or a new one.  Gradients that are zero because they have just been
+// passed on are known there too: they are read from one row of zeros, and not stored.
 //
-// M: two records per lane (one packed pair), one where the rows and the tape of two leave fewer than 12
+// A CTA is one warp, so that the walks' loops are uniform to the compiler: the operand records come
+// from the parameter space into uniform registers one section ahead, 32 bytes of ready offsets, and an
+// address is one register plus one uniform register.  (Records in shared memory took 2 of 3 of the walk's
+// shared-memory instructions; records packed into 16 bytes took a third more instructions.)
+//
+// M: two records per lane (one packed pair), one where the rows and slots of two leave fewer than 12
 // warps per SM (forward) or 8 (backward) in shared memory.  The walk's per-section work (operands,
 // branch, loop) is shared by a lane's records, but with four the warps that are left show the walk's
-// latency.  The forward pass gets 16 waves of CTAs, which evens out the SMs' distances from memory;
-// the backward pass is not bound by it.  Measured, 64 sections (23 of 24 fields written, 39 run
-// again, 14 tape values) over 2^24 records, one array per field:
-//   M         4                2                1
-//   forward   0.94 - 0.97 ms   0.91 (one wave: 1.00)   2.1     (64 section launches with saves: 2.8 ms)
-//   backward  3.07 ms          2.06 ms          2.58    (64 adjoint launches and a copy of the gradients: 6.1 ms)
-// What bounds it now: forward HBM at 0.78 of the copy bandwidth; backward the walk's chains of dependent
-// shared-memory loads and packed arithmetic at 12 warps per SM.  Operands from the parameter space
-// instead of shared memory one section ahead: 1.07 and 2.47 ms; two IEEE divisions per tanh pair
-// instead of tanh_pair's quotient: backward 2.24 ms.
+// latency.  16 waves of CTAs even out the SMs' distances from memory and the ends of their chunks
+// (backward with 1 wave 1.715 ms, 4 1.681, 8 1.655, 16 1.63).
+//
+// Measured, 64 sections (23 of 24 fields written, 39 run again, 9 slots beyond the fields') over 2^24
+// records, one array per field:
+//   forward   0.726 ms (64 section launches with saves: 2.8 ms); records in shared memory 0.910
+//   backward  1.63 ms (64 adjoint launches and a copy of the gradients: 6.1 ms); with a tape that old
+//             values were copied to and restored from, stored zeros and records in shared memory 2.060
+// What bounds it now: forward HBM, at 0.95 of the copy bandwidth; backward the walk's chains of dependent
+// shared-memory loads and packed arithmetic at 13 warps per SM (shared memory; issue active 0.55).
 #include <cuda_runtime.h>
 
 #include "internal.h"
@@ -40,11 +47,11 @@
 
 namespace adha {
 
-constexpr int kChainWarps = kChainThreads / 32;
-
-// Bytes of the tables before the warps' rows.
-__host__ __device__ __forceinline__ int chain_tables(const ChainArgs& a, bool backward) {
-  return a.n_rows * (int)sizeof(ChainRow) + (a.n_sec + (backward ? a.n_live : 0)) * (int)sizeof(ChainSec);
+// Bytes of the span lists before the warp's rows.
+__host__ __device__ __forceinline__ int chain_tables(const ChainArgs& a) {
+  int n = 0;
+  for (int k = 0; k < 4; ++k) n += a.n_span[k];
+  return n * (int)sizeof(ChainSpan);
 }
 
 // M floats of a lane as packed pairs (M = 1: the upper half is zero).
@@ -70,18 +77,13 @@ struct LaneVec {
   }
 };
 
-// One section on the lane's records (`s`: the lane's first record of row 0); TAPE: z's value from
-// before it goes to its tape slot, if it has one.
-template <int M, bool TAPE>
-__device__ __forceinline__ void chain_section(const ChainSec& c, uint8_t* s, uint8_t* tape, const unsigned long long* P,
+// One section on the lane's records (`s`: the lane's first record of row 0).
+template <int M>
+__device__ __forceinline__ void chain_section(const ChainSec& c, uint8_t* s, const unsigned long long* P,
                                               const unsigned long long* Q, unsigned long long nz) {
   constexpr int H = LaneVec<M>::H;
   LaneVec<M> x, v;
   x.load(s + c.x);
-  if (TAPE && c.tape >= 0) {
-    v.load(s + c.z);
-    v.store(tape + c.tape);
-  }
   if (c.op == ADHA_OP_AXPB) {
 #pragma unroll
     for (int h = 0; h < H; ++h) v.p[h] = f2_add_rn(f2_mul_alone(f2_pack(c.a, c.a), x.p[h], nz), f2_pack(c.b, c.b));
@@ -97,54 +99,39 @@ __device__ __forceinline__ void chain_section(const ChainSec& c, uint8_t* s, uin
   v.store(s + c.z);
 }
 
-// The adjoint of one section (adha_section_backward's rule, in its order): z restored from the tape,
-// gz = g[z], g[z] = 0, then g[x] (and g[y]) added to.  Every step goes through shared memory in
-// program order, so x, y and z may be the same field in any combination.
+// The adjoint of one section (adha_section_backward's rule, in its order): gz = g[z], g[z] = 0, then
+// g[x] (and g[y]) added to.  A zero is not stored: the planner knows which gradients are zero when and
+// has them read from the row of zeros; zero_rows says which are left so.
 template <int M>
-__device__ __forceinline__ void chain_adjoint(const ChainSec& c, uint8_t* s, uint8_t* g, const uint8_t* tape,
-                                              unsigned long long nz) {
+__device__ __forceinline__ void chain_adjoint(const ChainAdj& c, const uint8_t* s, uint8_t* g, unsigned long long nz) {
   constexpr int H = LaneVec<M>::H;
-  LaneVec<M> gz, gx, t, zero, old;
-#pragma unroll
-  for (int h = 0; h < H; ++h) zero.p[h] = 0ull;
-  gz.load(g + c.z);
-  zero.store(g + c.z);
-  gx.load(g + c.x);
+  LaneVec<M> gz, gx;
+  gz.load(g + c.gz);
+  gx.load(g + c.gx_in);
   if (c.op == ADHA_OP_AXPB) {
 #pragma unroll
     for (int h = 0; h < H; ++h) gx.p[h] = f2_add_rn(gx.p[h], f2_mul_alone(f2_pack(c.a, c.a), gz.p[h], nz));
-    gx.store(g + c.x);
-    if (c.tape >= 0) {
-      old.load(tape + c.tape);
-      old.store(s + c.z);
-    }
   } else if (c.op == ADHA_OP_TANH) {
-    t.load(s + c.z);   // the section's result: tanh(x)
+    LaneVec<M> t;
+    t.load(s + c.vx);
     const unsigned long long one = f2_pack(1.0f, 1.0f);
 #pragma unroll
     for (int h = 0; h < H; ++h)
       gx.p[h] = f2_add_rn(gx.p[h], f2_mul_alone(gz.p[h], f2_sub_rn(one, f2_mul_alone(t.p[h], t.p[h], nz)), nz));
-    gx.store(g + c.x);
-    if (c.tape >= 0) {
-      old.load(tape + c.tape);
-      old.store(s + c.z);
-    }
   } else {
     LaneVec<M> x, y, gy;
-    if (c.tape >= 0) {   // before x and y are read: either may be z
-      old.load(tape + c.tape);
-      old.store(s + c.z);
-    }
-    x.load(s + c.x);
-    y.load(s + c.y);
+    x.load(s + c.vx);
+    y.load(s + c.vy);
 #pragma unroll
     for (int h = 0; h < H; ++h) gx.p[h] = f2_add_rn(gx.p[h], f2_mul_alone(gz.p[h], y.p[h], nz));
-    gx.store(g + c.x);
-    gy.load(g + c.y);
+    gx.store(g + c.gx);
+    gy.load(g + c.gy_in);   // after the store: x and y may be the same field
 #pragma unroll
     for (int h = 0; h < H; ++h) gy.p[h] = f2_add_rn(gy.p[h], f2_mul_alone(gz.p[h], x.p[h], nz));
-    gy.store(g + c.y);
+    gy.store(g + c.gy);
+    return;
   }
+  gx.store(g + c.gx);
 }
 
 // Which of a row's addresses a load or store uses.
@@ -155,17 +142,28 @@ __device__ __forceinline__ uint8_t* row_base(const ChainRow& r) {
   return SIDE == kState ? r.state : SIDE == kGradIn ? const_cast<uint8_t*>(r.gin) : r.gout;
 }
 
-// Rows that are one contiguous array (one-field groups): 16-byte pieces, all rows in one walk.
-// FROM_SAVED: rows of written fields come from `saved` (contiguous whatever the layout), and rows
-// of wide groups that are not written are left to load_wide.
-template <int M, ChainSide SIDE, bool FROM_SAVED>
-__device__ __forceinline__ void load_rows(const ChainArgs& a, const ChainRow* rows, uint8_t* buf, int64_t i0, int lane) {
+// Contiguous arrays to rows or back, 16-byte pieces; a piece's place within its row depends on the lane
+// alone, so a piece costs one table load, one address addition and the copy.
+template <int M>
+__device__ __forceinline__ void load_spans(const ChainSpan* t, int n, uint8_t* buf, int64_t i0, int lane) {
   constexpr int PP = 8 * M;   // pieces per row
-  for (int p = lane; p < a.n_rows * PP; p += 32) {
-    const ChainRow& r = rows[p / PP];
-    const int q = (p % PP) * 16;
-    if (FROM_SAVED && r.saved >= 0) cp_async16(buf + p * 16, reinterpret_cast<const uint8_t*>(a.saved + r.saved * a.pitch + i0) + q);
-    else if (r.stride == 4) cp_async16(buf + p * 16, row_base<SIDE>(r) + i0 * 4 + q);
+  const int64_t from = i0 * 4 + lane % PP * 16;
+  uint8_t* to = buf + lane % PP * 16;
+#pragma unroll 2
+  for (int k = lane / PP; k < n; k += 32 / PP) {
+    const ChainSpan s = t[k];
+    cp_async16(to + s.at, s.base + from);
+  }
+}
+template <int M>
+__device__ __forceinline__ void store_spans(const ChainSpan* t, int n, const uint8_t* buf, int64_t i0, int lane) {
+  constexpr int PP = 8 * M;
+  const int64_t to = i0 * 4 + lane % PP * 16;
+  const uint8_t* from = buf + lane % PP * 16;
+#pragma unroll 2
+  for (int k = lane / PP; k < n; k += 32 / PP) {
+    const ChainSpan s = t[k];
+    *reinterpret_cast<uint4*>(s.base + to) = *reinterpret_cast<const uint4*>(from + s.at);
   }
 }
 
@@ -200,17 +198,12 @@ __device__ __forceinline__ void load_wide(const ChainArgs& a, const ChainRow* ro
   }
 }
 
-// Rows back to memory: contiguous rows in 16-byte pieces, wide groups lane = record.  WRITTEN: only
-// what the run writes (a wide group with a written field goes back whole where 16 bytes fit).
+// Rows of wide groups back to memory, lane = record.  WRITTEN: only what the run writes (a group with
+// a written field goes back whole where 16 bytes fit).
 template <int M, ChainSide SIDE, bool WRITTEN>
-__device__ __forceinline__ void store_rows(const ChainArgs& a, const ChainRow* rows, const uint8_t* buf, int64_t i0,
+__device__ __forceinline__ void store_wide(const ChainArgs& a, const ChainRow* rows, const uint8_t* buf, int64_t i0,
                                            int lane) {
-  constexpr int R = 32 * M, PP = 8 * M;
-  for (int p = lane; p < a.n_rows * PP; p += 32) {
-    const ChainRow& r = rows[p / PP];
-    if (r.stride == 4 && (!WRITTEN || r.saved >= 0))
-      *reinterpret_cast<uint4*>(row_base<SIDE>(r) + i0 * 4 + (p % PP) * 16) = *reinterpret_cast<const uint4*>(buf + p * 16);
-  }
+  constexpr int R = 32 * M;
   for (int k = 0; k < a.n_wide; ++k) {
     if (WRITTEN && !a.wide_written[k]) continue;
     const int row0 = a.wide_row[k], nf = a.wide_len[k], stride = rows[row0].stride;
@@ -263,31 +256,31 @@ __device__ __forceinline__ void store_tail(const ChainArgs& a, const ChainRow* r
   }
 }
 
-// The row table and the sections' operands in shared memory, one copy per CTA: the walks read an
-// operand block with two broadcast loads, one section ahead of its use.
-template <class T>
-__device__ __forceinline__ T* copy_table(const T* from, int n, uint8_t* to) {
-  static_assert(sizeof(T) % 16 == 0, "copied in 16-byte words");
-  for (int k = threadIdx.x; k < n * (int)(sizeof(T) / 16); k += kChainThreads)
-    reinterpret_cast<uint4*>(to)[k] = reinterpret_cast<const uint4*>(from)[k];
-  return reinterpret_cast<T*>(to);
+// Spans list l of the launch, copied to shared memory after the lists before it.
+__device__ __forceinline__ const ChainSpan* spans(const ChainArgs& a, int l, uint8_t* smem) {
+  int first = 0;
+  for (int k = 0; k < l; ++k) first += a.n_span[k];
+  ChainSpan* t = reinterpret_cast<ChainSpan*>(smem) + first;
+  for (int k = threadIdx.x; k < a.n_span[l]; k += kChainThreads) t[k] = a.span[l][k];
+  return t;
 }
 
 template <int M>
 __global__ void __launch_bounds__(kChainThreads) chain_forward_kernel(const __grid_constant__ ChainArgs a) {
   extern __shared__ __align__(16) uint8_t smem[];
-  constexpr int R = 32 * M, R4 = R * 4, PP = 8 * M;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const ChainRow* rows = copy_table(a.row, a.n_rows, smem);
-  const ChainSec* sec = copy_table(a.sec, a.n_sec, smem + a.n_rows * sizeof(ChainRow));
+  constexpr int R = 32 * M;
+  const int lane = threadIdx.x;
+  const ChainRow* rows = a.row;
+  const ChainSec* sec = a.sec;
+  const ChainSpan *in = spans(a, 0, smem), *save = spans(a, 1, smem), *out = spans(a, 2, smem);
   __syncthreads();
-  uint8_t* S = smem + chain_tables(a, false) + (size_t)warp * a.n_rows * R4;
+  uint8_t* S = smem + chain_tables(a);
   uint8_t* mine = S + lane * M * 4;
-  for (int64_t c = (int64_t)blockIdx.x * kChainWarps + warp; c < a.n_chunks; c += (int64_t)gridDim.x * kChainWarps) {
+  for (int64_t c = blockIdx.x; c < a.n_chunks; c += gridDim.x) {
     const int64_t i0 = c * R;
     const bool whole = i0 + R <= a.n;
     if (whole) {
-      load_rows<M, kState, false>(a, rows, S, i0, lane);
+      load_spans<M>(in, a.n_span[0], S, i0, lane);
       cp_async_commit();
       load_wide<M, kState, false>(a, rows, S, i0, lane);
       cp_async_wait<0>();
@@ -296,23 +289,22 @@ __global__ void __launch_bounds__(kChainThreads) chain_forward_kernel(const __gr
     }
     __syncwarp();
     // the written fields' values from before the run (rows of `saved` are padded to whole chunks)
-    for (int p = lane; p < a.n_rows * PP; p += 32) {
-      const int sv = rows[p / PP].saved;
-      if (sv >= 0)
-        *reinterpret_cast<uint4*>(reinterpret_cast<uint8_t*>(a.saved + sv * a.pitch + i0) + (p % PP) * 16) =
-            *reinterpret_cast<const uint4*>(S + p * 16);
-    }
+    store_spans<M>(save, a.n_span[1], S, i0, lane);
     __syncwarp();
     ChainSec next = sec[0];
 #pragma unroll 1
     for (int s = 0; s < a.n_sec; ++s) {
       const ChainSec c = next;
-      next = sec[min(s + 1, a.n_sec - 1)];
-      chain_section<M, false>(c, mine, nullptr, a.tanh_p, a.tanh_qn, a.neg_zero);
+      next = sec[s + 1];   // one beyond the last is never run
+      chain_section<M>(c, mine, a.tanh_p, a.tanh_qn, a.neg_zero);
     }
     __syncwarp();
-    if (whole) store_rows<M, kState, true>(a, rows, S, i0, lane);
-    else store_tail<M, kState, true>(a, rows, S, i0, lane);
+    if (whole) {
+      store_spans<M>(out, a.n_span[2], S, i0, lane);
+      store_wide<M, kState, true>(a, rows, S, i0, lane);
+    } else {
+      store_tail<M, kState, true>(a, rows, S, i0, lane);
+    }
     __syncwarp();
   }
 }
@@ -321,22 +313,26 @@ template <int M>
 __global__ void __launch_bounds__(kChainThreads) chain_backward_kernel(const __grid_constant__ ChainArgs a) {
   extern __shared__ __align__(16) uint8_t smem[];
   constexpr int R = 32 * M, R4 = R * 4;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const ChainRow* rows = copy_table(a.row, a.n_rows, smem);
-  const ChainSec* sec = copy_table(a.sec, a.n_sec, smem + a.n_rows * sizeof(ChainRow));
-  const ChainSec* live = copy_table(a.live, a.n_live, smem + a.n_rows * sizeof(ChainRow) + a.n_sec * sizeof(ChainSec));
+  const int lane = threadIdx.x;
+  const ChainRow* rows = a.row;
+  const ChainSec* live = a.sec;
+  const ChainAdj* adj = a.adj;
+  const ChainSpan *in = spans(a, 0, smem), *out = spans(a, 1, smem), *gin = spans(a, 2, smem), *gout = spans(a, 3, smem);
   __syncthreads();
-  uint8_t* S = smem + chain_tables(a, true) + (size_t)warp * (2 * a.n_rows + a.n_tape) * R4;
-  uint8_t* G = S + a.n_rows * R4;
-  uint8_t* T = G + a.n_rows * R4;
+  uint8_t* S = smem + chain_tables(a);
+  uint8_t* G = S + (a.n_rows + a.n_tape) * R4;
   const int at = lane * M * 4;
-  for (int64_t c = (int64_t)blockIdx.x * kChainWarps + warp; c < a.n_chunks; c += (int64_t)gridDim.x * kChainWarps) {
+  LaneVec<M> zero;
+#pragma unroll
+  for (int h = 0; h < LaneVec<M>::H; ++h) zero.p[h] = 0ull;
+  zero.store(G + a.n_rows * R4 + at);   // the row of zeros
+  for (int64_t c = blockIdx.x; c < a.n_chunks; c += gridDim.x) {
     const int64_t i0 = c * R;
     const bool whole = i0 + R <= a.n;
     if (whole) {
-      load_rows<M, kState, true>(a, rows, S, i0, lane);
+      load_spans<M>(in, a.n_span[0], S, i0, lane);
       cp_async_commit();
-      load_rows<M, kGradIn, false>(a, rows, G, i0, lane);   // arrives while the sections run again
+      load_spans<M>(gin, a.n_span[2], G, i0, lane);   // arrives while the sections run again
       cp_async_commit();
       load_wide<M, kState, true>(a, rows, S, i0, lane);
       load_wide<M, kGradIn, false>(a, rows, G, i0, lane);
@@ -347,28 +343,37 @@ __global__ void __launch_bounds__(kChainThreads) chain_backward_kernel(const __g
     }
     __syncwarp();
     // the state as it was before the run
-    if (whole) store_rows<M, kState, true>(a, rows, S, i0, lane);
-    else store_tail<M, kState, true>(a, rows, S, i0, lane);
+    if (whole) {
+      store_spans<M>(out, a.n_span[1], S, i0, lane);
+      store_wide<M, kState, true>(a, rows, S, i0, lane);
+    } else {
+      store_tail<M, kState, true>(a, rows, S, i0, lane);
+    }
     __syncwarp();
     ChainSec next = live[0];
 #pragma unroll 1
     for (int s = 0; s < a.n_live; ++s) {
       const ChainSec c = next;
-      next = live[min(s + 1, a.n_live - 1)];
-      chain_section<M, true>(c, S + at, T + at, a.tanh_p, a.tanh_qn, a.neg_zero);
+      next = live[s + 1];
+      chain_section<M>(c, S + at, a.tanh_p, a.tanh_qn, a.neg_zero);
     }
-    next = sec[a.n_sec - 1];
+    ChainAdj nadj = adj[0];
     cp_async_wait<0>();
     __syncwarp();
 #pragma unroll 1
-    for (int s = a.n_sec - 1; s >= 0; --s) {
-      const ChainSec c = next;
-      next = sec[max(s - 1, 0)];
-      chain_adjoint<M>(c, S + at, G + at, T + at, a.neg_zero);
+    for (int s = 0; s < a.n_sec; ++s) {
+      const ChainAdj c = nadj;
+      nadj = adj[s + 1];
+      chain_adjoint<M>(c, S + at, G + at, a.neg_zero);
     }
+    for (uint64_t left = a.zero_rows; left; left &= left - 1) zero.store(G + (__ffsll((long long)left) - 1) * R4 + at);
     __syncwarp();
-    if (whole) store_rows<M, kGradOut, false>(a, rows, G, i0, lane);
-    else store_tail<M, kGradOut, false>(a, rows, G, i0, lane);
+    if (whole) {
+      store_spans<M>(gout, a.n_span[3], G, i0, lane);
+      store_wide<M, kGradOut, false>(a, rows, G, i0, lane);
+    } else {
+      store_tail<M, kGradOut, false>(a, rows, G, i0, lane);
+    }
     // gradients of groups the run does not touch, when they go to buffers of their own
     for (int k = 0; k < a.n_copy; ++k) {
       const ChainCopy& cp = a.copy[k];
@@ -382,7 +387,7 @@ __global__ void __launch_bounds__(kChainThreads) chain_backward_kernel(const __g
 }
 
 size_t chain_smem_bytes(const ChainArgs& a, int M, bool backward) {
-  return chain_tables(a, backward) + (size_t)kChainWarps * (backward ? 2 * a.n_rows + a.n_tape : a.n_rows) * 128 * M;
+  return chain_tables(a) + (size_t)(backward ? 2 * a.n_rows + a.n_tape + 1 : a.n_rows) * 128 * M;
 }
 
 template <class K>

@@ -159,8 +159,8 @@ struct BackwardArgs {
 // A run of fp32 chain sections and its gradient in one pass each (chain.cu).  Rows are the fields of
 // every group that a section of the run touches, a group's fields consecutive.
 constexpr int kMaxChain = 128;       // sections in one run
-constexpr int kMaxChainTape = 96;    // overwritten values a run's reverse walk may need
-constexpr int kChainThreads = 64;    // small CTAs: a warp's rows take 10-30 KB, so whole CTAs waste less
+constexpr int kMaxChainTape = 96;    // values beyond one per field that a run's reverse walk may hold
+constexpr int kChainThreads = 32;    // one warp per CTA: its loops are uniform to the compiler (see chain.cu)
 struct ChainRow {
   uint8_t* state;        // the field in record 0
   const uint8_t* gin;    // its gradient (backward)
@@ -168,30 +168,48 @@ struct ChainRow {
   int32_t stride;        // the group's struct size; 4: the row is one contiguous array
   int32_t saved;         // its row of `saved` if the run writes it, else -1
 };
+// One section to run: byte offsets of its operands' rows, or in the backward pass of the slots that
+// hold them.
 struct __align__(16) ChainSec {
-  int32_t op, x, y, z;   // operand rows, as byte offsets for the launch's chunk
+  int32_t op, x, y, z;
   float a, b;            // AXPB
-  int32_t tape;          // byte offset of the tape slot for z's value from before the section, -1 if the reverse
-                         // walk does not need it
-  int32_t pad;
+  int32_t pad[2];
+};
+// The adjoint of one section: byte offsets of the gradient rows of z, x and y (the row of zeros where a
+// gradient that is read is zero at this point), and of the values that it multiplies by.
+struct __align__(16) ChainAdj {
+  int32_t op, gz, gx_in, gx;
+  int32_t gy_in, gy;
+  union {
+    float a;             // AXPB
+    int32_t vx;          // MUL: x as it was before the section; TANH: the section's result
+  };
+  int32_t vy;            // MUL: y as it was before the section
 };
 struct ChainCopy {       // a group the run does not touch whose gradient goes to a buffer of its own
   const uint8_t* src;
   uint8_t* dst;
   int32_t stride;
 };
+struct ChainSpan {       // an array of 4-byte values that one row of a chunk comes from or goes to
+  uint8_t* base;         // record 0
+  int32_t at, pad;       // the row's byte offset
+};
 struct ChainArgs {
   int64_t n, n_chunks;   // records; chunks counting the ragged one
   int64_t pitch;         // floats per row of `saved`: n rounded up to whole 128-record chunks
   float* saved;
   unsigned long long neg_zero;   // the pair (-0, -0) (see f2_mul_alone)
-  int32_t n_rows, n_sec, n_live, n_tape, n_wide, n_copy;
+  int32_t n_rows, n_sec, n_live, n_tape, n_wide, n_copy;   // n_sec: sections of `sec` or `adj`; n_tape: slots beyond the rows
+  uint64_t zero_rows;    // gradient rows that are zero after the reverse walk
   unsigned long long tanh_p[8], tanh_qn[8];   // the coefficients of P and -Q as pairs
   int8_t wide_row[kMaxFields], wide_len[kMaxFields], wide_written[kMaxFields];   // groups of two or more fields
   ChainRow row[kMaxFields];
+  int32_t n_span[4];
+  ChainSpan span[4][kMaxFields];   // forward: rows in, saved, out; backward: rows in, out, gradients in, out
   ChainCopy copy[kMaxGroups];
-  ChainSec sec[kMaxChain];    // the run's sections
-  ChainSec live[kMaxChain];   // those that the backward pass runs again
+  ChainSec sec[kMaxChain + 1];    // the sections to run: all, or (n_live) those that the backward pass runs again
+  ChainAdj adj[kMaxChain + 1];    // backward: every section's adjoint, in the reverse walk's order
 };
 
 // Plan + launch helpers shared by the entry points, the measurer and the executor.
