@@ -332,6 +332,14 @@ static int finish_grid(int64_t n_chunks, int blocks, int* grid) {
   return 0;
 }
 
+// Waves of CTAs for kernels that even out the SMs with more than one: no more than leave every warp
+// `least` chunks, or a CTA's set-up costs more than the evening out gives.  2^20 records: arrays into
+// 80-byte structs 28.7 -> 23.2 us, assign 49 -> 41, 80-byte structs to arrays (least 1) 33.4 -> 30.7; the
+// same as without the limit from 2^23 records on.
+static int waves_for(int64_t n_chunks, int sms, int resident_warps, int waves, int least) {
+  return (int)std::max<int64_t>(1, std::min<int64_t>(waves, n_chunks / std::max<int64_t>(1, (int64_t)sms * resident_warps * least)));
+}
+
 // Shared-memory wavefronts of one warp step (32 schedule entries of one move class): the
 // largest number of distinct 4-byte words that fall in one bank, for the given byte addresses.
 static int step_wavefronts(const uint32_t* bytes, int cnt, int width) {
@@ -706,7 +714,7 @@ static int plan_columns(const Layout& S, const void* const* src_ptrs, const Layo
   int blocks = 0;
   if (int rc = cached_occupancy(100 + (R == 128 ? 2 : R == 64 ? 1 : 0), plan->smem, &blocks)) return rc;
   *fits = true;
-  return finish_grid(a.n_chunks, blocks * waves, &plan->grid);
+  return finish_grid(a.n_chunks, blocks * waves_for(a.n_chunks, sms, blocks * kWarps, waves, out_rec ? 2 : 1), &plan->grid);
 }
 
 // ------------------------------------------------------------------ section planning
@@ -980,7 +988,10 @@ static int plan_section(const Layout& L, void* const* ptrs, const adha_section* 
   int blocks = 0;
   if (int rc = cached_occupancy(1000 + 1000 * s->op + a.R + a.vec, plan->smem, &blocks)) return rc;
   // assign has little to set up per CTA and its stores are uneven work: 280 us in one wave, 262 at 8
-  return finish_grid(a.n_chunks, blocks * (s->op == ADHA_OP_ASSIGN ? 8 : 1), &plan->grid);
+  int waves = 1, sms = 0;
+  if (int rc = sm_count(&sms)) return rc;
+  if (s->op == ADHA_OP_ASSIGN) waves = waves_for(a.n_chunks, sms, blocks * kWarps, 8, 2);
+  return finish_grid(a.n_chunks, blocks * waves, &plan->grid);
 }
 
 int remap_plan_args(const Layout& S, const void* const* src_ptrs, const Layout& D, void* const* dst_ptrs, int64_t n,
@@ -1263,7 +1274,9 @@ static int plan_fused(const Layout& L, void* const* ptrs, const adha_section* s,
       if (int e = jit_occupancy(fn, plan->smem, &blocks)) return e;
       // nothing to set up per CTA: many short CTAs even out the SMs' distances from memory (nine
       // stress sections one by one, 2^24 records: 1997 us in one wave, 1879 at 4, 1796 at 16)
-      return finish_grid(a.n_chunks, blocks * 16, &plan->grid);
+      int sms = 0;
+      if (int e = sm_count(&sms)) return e;
+      return finish_grid(a.n_chunks, blocks * waves_for(a.n_chunks, sms, blocks * kWarps, 16, 1), &plan->grid);
     }
     if (t_fused_jit == 2) return rc;   // asked for explicitly: report why not
     clear_error();                     // else the library's fused kernel
@@ -1543,7 +1556,7 @@ static int run_chain(const Layout& L, void* const* ptrs, const void* const* gin,
   int blocks = 0;
   if (int rc = cached_occupancy(300 + 10 * M + (backward ? 1 : 0), smem, &blocks)) return rc;
   if (blocks < 1) return fail(ADHA_ENOTIMPL, "kernel does not fit on an SM");
-  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)sms * blocks * 16, a.n_chunks));
+  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)sms * blocks * waves_for(a.n_chunks, sms, blocks, 16, 1), a.n_chunks));
   const int n_saved = __builtin_popcountll(written), n_touched = __builtin_popcountll(touched);
   // what the pass has to move: the touched fields in, the written ones out and saved; backward the
   // gradients in and out, the saved values in, and the state back
