@@ -211,9 +211,8 @@ __global__ void __launch_bounds__(kThreads) fused_kernel(const __grid_constant__
     }
   }
   if constexpr (KM) {
-    if (a.reduce_sec >= 0) {   // every warp adds its sums and counts into the result
-      __syncwarp();
-      reduce_flush(rq, secs[a.reduce_sec], lane, acc, sum, &cnt_lane);
+    if (a.reduce_sec >= 0) {   // the CTA adds its sums and counts into the result
+      reduce_flush(rq, secs[a.reduce_sec], warp, lane, reinterpret_cast<long long*>(idx - warp * kReduceList), acc, sum, &cnt_lane);
     }
   }
 }

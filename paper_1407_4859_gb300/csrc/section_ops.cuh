@@ -999,21 +999,28 @@ __device__ __forceinline__ void reduce_tail(const ReduceLane& q, const SecOp& so
   }
 }
 
-// The warp's sums and counts added into the result (K rows of [count, d sums], zeroed before
-// the launch unless the caller accumulates).
-__device__ __forceinline__ void reduce_flush(const ReduceLane& q, const SecOp& so, int lane, const long long* acc,
-                                             const long long (&sum)[kMaxClusters], const unsigned long long* cnt) {
-  unsigned long long* out = static_cast<unsigned long long*>(const_cast<void*>(so.aux));
-  const int d = q.d;
+// The warps' sums and counts into the result, by all threads of the CTA: added up in shared memory
+// first (`table`: the CTA's record lists, done with by now), or 1.3 million additions to a few hundred
+// addresses would be most of a short launch.  Whole numbers: the order does not matter.
+__device__ __forceinline__ void reduce_flush(const ReduceLane& q, const SecOp& so, int warp, int lane, long long* table,
+                                             const long long* acc, const long long (&sum)[kMaxClusters],
+                                             const unsigned long long* cnt) {
+  static_assert(kReduceListBytes >= kMaxClusters * 33 * 8, "the table fits the record lists");
+  const int d = q.d, row = d + 1;
+  for (int w = 0; w < kWarps; ++w) {
+    __syncthreads();
+    if (warp != w) continue;
 #pragma unroll
-  for (int k = 0; k < kMaxClusters; ++k)
-    if (k < q.K) {
-      if (lane < d) {
+    for (int k = 0; k < kMaxClusters; ++k)
+      if (k < q.K && lane < d) {
         const long long v = q.walk ? sum[k] : acc[k * 32 + lane] + acc[(kMaxClusters + 1 + k) * 32 + lane];
-        atomicAdd(out + (size_t)k * (d + 1) + 1 + lane, (unsigned long long)v);
+        table[k * row + 1 + lane] = w ? table[k * row + 1 + lane] + v : v;
       }
-    }
-  if (lane < q.K) atomicAdd(out + (size_t)lane * (d + 1), *cnt);
+    if (lane < q.K) table[lane * row] = (w ? table[lane * row] : 0) + (long long)*cnt;
+  }
+  __syncthreads();
+  unsigned long long* out = static_cast<unsigned long long*>(const_cast<void*>(so.aux));
+  for (int e = warp * 32 + lane; e < q.K * row; e += kThreads) atomicAdd(out + e, (unsigned long long)table[e]);
 }
 
 }  // namespace adha

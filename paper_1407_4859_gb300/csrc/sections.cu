@@ -151,9 +151,8 @@ __global__ void __launch_bounds__(kThreads) section_kernel(const __grid_constant
   const int64_t t0 = a.n_chunks * R;
   if constexpr (OP == ADHA_OP_REDUCE) {
     if (c == a.n_chunks && t0 < a.n) reduce_tail(rq, a.s, a.f, t0, a.n, lane, acc, sum, &cnt);
-    // every warp adds its sums and counts into the result (zeroed before the launch)
-    __syncwarp();
-    reduce_flush(rq, a.s, lane, acc, sum, &cnt);
+    // the CTA adds its sums and counts into the result (zeroed before the launch)
+    reduce_flush(rq, a.s, warp, lane, reinterpret_cast<long long*>(idx - warp * kReduceList), acc, sum, &cnt);
   } else {
     if (c == a.n_chunks && t0 < a.n) {
       for (int64_t i = t0 + lane; i < a.n; i += 32)
