@@ -115,7 +115,7 @@ KERNEL_SOURCES = {
     "specialised": ["jit.cu", "fused_jit.cuh", "section_ops.cuh", "device_types.h", "ptx.cuh"],
     "section": ["sections.cu", "section_ops.cuh", "staging.cuh", "device_types.h", "ptx.cuh"],
     "section_backward": ["sections.cu", "section_ops.cuh", "device_types.h"],
-    "remap": ["remap.cu", "remap_common.cuh", "internal.h", "ptx.cuh"],
+    "remap": ["remap.cu", "remap_common.cuh", "staging.cuh", "internal.h", "ptx.cuh"],
     "batched_remap": ["batched.cu", "remap_common.cuh", "internal.h", "ptx.cuh"],
     "fused": ["fused.cu", "section_ops.cuh", "staging.cuh", "device_types.h", "ptx.cuh"],
     "chain": ["chain.cu", "section_ops.cuh", "internal.h", "ptx.cuh"],

@@ -648,8 +648,7 @@ static int plan_columns(const Layout& S, const void* const* src_ptrs, const Layo
     waves = several ? 1 : 8;
     table = several;
   }
-  const int nb = 1;
-  auto warp_bytes = [&](int r) { return r * (nb * in_rec + out_rec); };
+  auto warp_bytes = [&](int r) { return r * (in_rec + out_rec); };
   int sms = 0;
   if (int rc = sm_count(&sms)) return rc;
   while (R > 32 && n < (int64_t)R * sms * 8) R /= 2;   // few records: chunks for every SM
@@ -660,7 +659,6 @@ static int plan_columns(const Layout& S, const void* const* src_ptrs, const Layo
   a.R = R;
   a.n_chunks = n / R;
   if (a.n_chunks >> 32) return 0;   // chunk numbers are 32-bit in the address arithmetic
-  a.buffers = nb;
   a.fill = padding ? 1 : 0;
   int in_at[kMaxGroups], off = 0;
   for (int j : need) {
@@ -1421,11 +1419,11 @@ static uint64_t chain_read(const adha_section* s, int m) {
   return r;
 }
 
-// Leading sections of s[0..m) that fit one run: at most kMaxChain, and at most kMaxChainTape slots
+// Leading sections of s[0..m) that fit one run: at most kMaxChain, and at most kMaxChainExtra slots
 // beyond the fields' own (with the rows of 64 fields and their gradients, eight warps per SM).
 static int chain_window(int F, const adha_section* s, int m) {
   int k = std::min(m, kMaxChain);
-  while (k > 1 && chain_slots(F, chain_written(s, k) | chain_read(s, k), s, k).extra > kMaxChainTape) k = std::max(1, k - 8);
+  while (k > 1 && chain_slots(F, chain_written(s, k) | chain_read(s, k), s, k).extra > kMaxChainExtra) k = std::max(1, k - 8);
   return k;
 }
 
@@ -1486,9 +1484,9 @@ static int run_chain(const Layout& L, void* const* ptrs, const void* const* gin,
   }
   ChainSlots slots;
   if (backward) slots = chain_slots(L.F, rows, s, m);
-  a.n_tape = slots.extra;
+  a.n_extra = slots.extra;
   // records per lane: two, fewer where that leaves less than 12 (forward) or 8 (backward) warps per SM
-  const int per_warp = 128 * (backward ? 2 * a.n_rows + a.n_tape + 1 : a.n_rows), warps = backward ? 8 : 12;
+  const int per_warp = 128 * (backward ? 2 * a.n_rows + a.n_extra + 1 : a.n_rows), warps = backward ? 8 : 12;
   int M = 2;
   while (M > 1 && (size_t)warps * M * per_warp > kSmemPerSM - 16 * 1024) M /= 2;
   // few records: short chunks, so that every SM has work

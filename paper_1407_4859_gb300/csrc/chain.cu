@@ -320,7 +320,7 @@ __global__ void __launch_bounds__(kChainThreads) chain_backward_kernel(const __g
   const ChainSpan *in = spans(a, 0, smem), *out = spans(a, 1, smem), *gin = spans(a, 2, smem), *gout = spans(a, 3, smem);
   __syncthreads();
   uint8_t* S = smem + chain_tables(a);
-  uint8_t* G = S + (a.n_rows + a.n_tape) * R4;
+  uint8_t* G = S + (a.n_rows + a.n_extra) * R4;
   const int at = lane * M * 4;
   LaneVec<M> zero;
 #pragma unroll
@@ -387,7 +387,7 @@ __global__ void __launch_bounds__(kChainThreads) chain_backward_kernel(const __g
 }
 
 size_t chain_smem_bytes(const ChainArgs& a, int M, bool backward) {
-  return chain_tables(a) + (size_t)(backward ? 2 * a.n_rows + a.n_tape + 1 : a.n_rows) * 128 * M;
+  return chain_tables(a) + (size_t)(backward ? 2 * a.n_rows + a.n_extra + 1 : a.n_rows) * 128 * M;
 }
 
 template <class K>

@@ -110,7 +110,6 @@ struct ColumnArgs {
   int32_t R;               // 32, 64 or 128; 8 or 16 for wide records
   int32_t n_in, n_out;     // slices
   int32_t in_bytes, out_bytes;
-  int32_t buffers;         // chunk buffers per warp: 2 (the next chunk copied in during this one) or 1
   int32_t fill;            // 1: destination structs have padding (zeroed once, never written)
   int32_t n_pieces;        // > 0: the input's 16-byte pieces through a table of that many (staging.cuh)
   int32_t cnt[kColClasses];
@@ -159,7 +158,7 @@ struct BackwardArgs {
 // A run of fp32 chain sections and its gradient in one pass each (chain.cu).  Rows are the fields of
 // every group that a section of the run touches, a group's fields consecutive.
 constexpr int kMaxChain = 128;       // sections in one run
-constexpr int kMaxChainTape = 96;    // values beyond one per field that a run's reverse walk may hold
+constexpr int kMaxChainExtra = 96;    // values beyond one per field that a run's reverse walk may hold
 constexpr int kChainThreads = 32;    // one warp per CTA: its loops are uniform to the compiler (see chain.cu)
 struct ChainRow {
   uint8_t* state;        // the field in record 0
@@ -200,7 +199,7 @@ struct ChainArgs {
   int64_t pitch;         // floats per row of `saved`: n rounded up to whole 128-record chunks
   float* saved;
   unsigned long long neg_zero;   // the pair (-0, -0) (see f2_mul_alone)
-  int32_t n_rows, n_sec, n_live, n_tape, n_wide, n_copy;   // n_sec: sections of `sec` or `adj`; n_tape: slots beyond the rows
+  int32_t n_rows, n_sec, n_live, n_extra, n_wide, n_copy;   // n_sec: sections of `sec` or `adj`; n_extra: slots beyond the rows
   uint64_t zero_rows;    // gradient rows that are zero after the reverse walk
   unsigned long long tanh_p[8], tanh_qn[8];   // the coefficients of P and -Q as pairs
   int8_t wide_row[kMaxFields], wide_len[kMaxFields], wide_written[kMaxFields];   // groups of two or more fields

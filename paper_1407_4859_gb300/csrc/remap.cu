@@ -1,8 +1,10 @@
 // remap.cu -- the layout remap kernel (paper Section 2: the remap between two sections' layouts;
 // Table 4: CPU-ODS(1-3) remap GPU-ODS(4-7)).
 //
-// Every warp works alone on chunks of R consecutive records (R a multiple of 32), so the main
-// loop has no block-wide barrier:
+// Two kernels: column_kernel, lane = record, the default (described below), and remap_kernel, by an
+// element schedule, for tuned or forced shapes and records too wide for the other.  In both every warp
+// works alone on chunks of R consecutive records, so that the main loop has no block-wide barrier.
+// remap_kernel (R a multiple of 8):
 //   1. the warp copies the chunk's slice of every source group into its own shared buffer with
 //      16-byte cp.async (coalesced: lane l moves bytes 16l, 16l+512, ...): one chunk ahead of
 //      the one it works on (two buffers), or, with one buffer, as soon as the moves have read
@@ -146,9 +148,8 @@ struct Columns {
   const StagePiece* tab;   // the input pieces of a chunk, NULL: slice by slice
   int n_pieces;
   int R, lane;
-  uint8_t *ibuf, *obuf;   // the warp's input buffers and its output buffer
+  uint8_t *ibuf, *obuf;   // the warp's buffers
 
-  __device__ __forceinline__ uint8_t* ib(int b) const { return ibuf + b * a.in_bytes; }
   __device__ __forceinline__ bool on(int m, int cnt) const { return lane + 32 * m < cnt; }
 
   // Places of the 16-byte pieces of `bytes` bytes of a slice: f(piece offset in memory, in the buffer).
@@ -161,11 +162,11 @@ struct Columns {
     }
   }
 
-  // The chunk's source slices into buffer b.
+  // The chunk's source slices into the input buffer.
   template <bool WHOLE>
-  __device__ __forceinline__ void stage(int64_t ch, int b, int cnt) const {
-    if (WHOLE && tab) return stage_chunk(tab, n_pieces, ch, ib(b), lane);
-    const uint32_t si = smem_addr(ib(b));
+  __device__ __forceinline__ void stage(int64_t ch, int cnt) const {
+    if (WHOLE && tab) return stage_chunk(tab, n_pieces, ch, ibuf, lane);
+    const uint32_t si = smem_addr(ibuf);
     for (int k = 0; k < a.n_in; ++k) {
       const ColSlice s = in[k];
       const int stride = s.stride & kColStride, bytes = cnt * stride;
@@ -215,9 +216,9 @@ struct Columns {
   }
 
   template <bool WHOLE>
-  __device__ __forceinline__ void moves(int64_t ch, int b, int cnt) const {
+  __device__ __forceinline__ void moves(int64_t ch, int cnt) const {
     const int64_t i0 = ch * R;
-    const uint8_t* src = ib(b);
+    const uint8_t* src = ibuf;
     int k = 0, e = a.cnt[0];
     column_out<unsigned long long, WHOLE>(k, e, src, i0, cnt);
     k = e, e += a.cnt[1];
@@ -234,12 +235,12 @@ struct Columns {
 
   // The built (or carried) structs of the chunk to memory.
   template <bool WHOLE>
-  __device__ __forceinline__ void write_out(int64_t ch, int b, int cnt) const {
+  __device__ __forceinline__ void write_out(int64_t ch, int cnt) const {
     for (int k = 0; k < a.n_out; ++k) {
       const ColSlice s = out[k];
       const int stride = s.stride & kColStride, bytes = cnt * stride;
       uint8_t* dst = const_cast<uint8_t*>(s.ptr) + (uint64_t)(uint32_t)ch * (uint32_t)(R * stride);
-      const uint8_t* src = (s.stride & kColFromIn ? ib(b) : obuf) + s.at;
+      const uint8_t* src = (s.stride & kColFromIn ? ibuf : obuf) + s.at;
       pieces(s, bytes, [&](int p, int at) {
         if (WHOLE || p + 16 <= bytes) {
           *reinterpret_cast<uint4*>(dst + p) = *reinterpret_cast<const uint4*>(src + at);
@@ -258,7 +259,6 @@ __global__ void __launch_bounds__(kThreads, 4) column_kernel(const __grid_consta
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   int n_col = 0;
   for (int k = 0; k < kColClasses; ++k) n_col += a.cnt[k];
-  const int nb = a.buffers;
   ColMove* col = reinterpret_cast<ColMove*>(smem);
   ColSlice* in = reinterpret_cast<ColSlice*>(col + n_col);
   ColSlice* out = in + a.n_in;
@@ -274,41 +274,34 @@ __global__ void __launch_bounds__(kThreads, 4) column_kernel(const __grid_consta
     const int room = a.in[k].stride & kColRoom ? 16 * (int)__umulhi((unsigned)p, a.in[k].magic) : 0;
     tab[q] = StagePiece{a.in[k].ptr + p, R * stride, a.in[k].at + p + room};
   }
-  uint8_t* mine = reinterpret_cast<uint8_t*>(tab + a.n_pieces) + (size_t)warp * (nb * a.in_bytes + a.out_bytes);
+  uint8_t* mine = reinterpret_cast<uint8_t*>(tab + a.n_pieces) + (size_t)warp * (a.in_bytes + a.out_bytes);
   if (a.fill)
     for (int p = lane * 16; p < a.out_bytes; p += 512)
-      *reinterpret_cast<uint4*>(mine + nb * a.in_bytes + p) = make_uint4(0, 0, 0, 0);
+      *reinterpret_cast<uint4*>(mine + a.in_bytes + p) = make_uint4(0, 0, 0, 0);
   __syncthreads();
-  const Columns<M> w{a, col, in, out, a.n_pieces ? tab : nullptr, a.n_pieces, R, lane, mine, mine + nb * a.in_bytes};
+  const Columns<M> w{a, col, in, out, a.n_pieces ? tab : nullptr, a.n_pieces, R, lane, mine, mine + a.in_bytes};
   const int64_t W = (int64_t)gridDim.x * kWarps;
-  // one input buffer: the next chunk may come in once the moves have read this one, unless groups are
-  // written from it
-  bool early = nb == 1;
+  // the next chunk may come in once the moves have read this one, unless groups are written from it
+  bool early = true;
   for (int k = 0; k < a.n_out; ++k) early = early && !(out[k].stride & kColFromIn);
 
   int64_t c = (int64_t)blockIdx.x * kWarps + warp;
-  if (c < a.n_chunks) w.template stage<true>(c, 0, R);
+  if (c < a.n_chunks) w.template stage<true>(c, R);
   cp_async_commit();
-  for (int i = 0; c < a.n_chunks; c += W, i ^= nb - 1) {
+  for (; c < a.n_chunks; c += W) {
     const bool more = c + W < a.n_chunks;
-    if (nb == 2) {
-      if (more) w.template stage<true>(c + W, i ^ 1, R);
-      cp_async_commit();
-      cp_async_wait<1>();
-    } else {
-      cp_async_wait<0>();
-    }
+    cp_async_wait<0>();
     __syncwarp();
-    w.template moves<true>(c, i, R);
+    w.template moves<true>(c, R);
     __syncwarp();
     if (early && more) {
-      w.template stage<true>(c + W, 0, R);
+      w.template stage<true>(c + W, R);
       cp_async_commit();
     }
-    w.template write_out<true>(c, i, R);
+    w.template write_out<true>(c, R);
     __syncwarp();
-    if (nb == 1 && !early && more) {
-      w.template stage<true>(c + W, 0, R);
+    if (!early && more) {
+      w.template stage<true>(c + W, R);
       cp_async_commit();
     }
   }
@@ -317,13 +310,13 @@ __global__ void __launch_bounds__(kThreads, 4) column_kernel(const __grid_consta
   if (c == a.n_chunks && rest > 0) {
     cp_async_wait<0>();
     __syncwarp();
-    w.template stage<false>(c, 0, rest);
+    w.template stage<false>(c, rest);
     cp_async_commit();
     cp_async_wait<0>();
     __syncwarp();
-    w.template moves<false>(c, 0, rest);
+    w.template moves<false>(c, rest);
     __syncwarp();
-    w.template write_out<false>(c, 0, rest);
+    w.template write_out<false>(c, rest);
   }
   cp_async_wait<0>();
 }
@@ -331,7 +324,7 @@ __global__ void __launch_bounds__(kThreads, 4) column_kernel(const __grid_consta
 size_t columns_smem_bytes(const ColumnArgs& a) {
   int n_col = 0;
   for (int k = 0; k < kColClasses; ++k) n_col += a.cnt[k];
-  return (size_t)(n_col + a.n_in + a.n_out + a.n_pieces) * 16 + (size_t)kWarps * ((size_t)a.buffers * a.in_bytes + a.out_bytes);
+  return (size_t)(n_col + a.n_in + a.n_out + a.n_pieces) * 16 + (size_t)kWarps * ((size_t)a.in_bytes + a.out_bytes);
 }
 
 template <int M>
