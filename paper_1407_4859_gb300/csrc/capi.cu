@@ -903,10 +903,12 @@ static int plan_section(const Layout& L, void* const* ptrs, const adha_section* 
     if (R == 96) R = 64;
   }
   if (!tuned_R) {
-    // few records: shorter chunks, so that every SM's schedulers have a warp
+    // few records: shorter chunks, so that every SM's schedulers have a warp; a reduce takes its chunk's
+    // records one after another, and gains from 24 chunks per SM (151651 records of 12 bytes 20.9 -> 13.3
+    // us, 343024 of 56 bytes 31.6 -> 21.4)
     int sms = 0;
     if (int rc = sm_count(&sms)) return rc;
-    while (R > 32 && n < (int64_t)R * sms * 4) R /= 2;
+    while (R > 32 && n < (int64_t)R * sms * (s->op == ADHA_OP_REDUCE ? 24 : 4)) R /= 2;
   }
   if (buffers != 1) buffers = 2;
   if (n >> 36) R = 128;   // chunk numbers below 2^32 (so many records are a few bytes each: 128 of them fit)
@@ -1192,8 +1194,11 @@ static int plan_fused(const Layout& L, void* const* ptrs, const adha_section* s,
   if (tuned_R) R = std::max(32, std::min(tuned_R, 128));
   else if (one_field && (size_t)kWarps * 2 * 128 * rec <= (size_t)kSmemLimit / 2 - 8192) R = 128;
   else if (one_field && (size_t)kWarps * 2 * 64 * rec <= (size_t)kSmemLimit / 2 - 8192) R = 64;
-  else if (reduce_sec >= 0 || assign_sec >= 0) R = 64;   // as the sections by themselves (plan_section)
-  else R = rec > 0 ? pick_chunk(rec, 4096, 128) : 128;
+  else if (reduce_sec >= 0 || assign_sec >= 0) {   // as the sections by themselves (plan_section)
+    int sms = 0;
+    if (int rc = sm_count(&sms)) return rc;
+    R = n < (int64_t)64 * sms * 8 ? 32 : 64;   // 11197 records of 52 bytes: 23.3 -> 17.4 us
+  } else R = rec > 0 ? pick_chunk(rec, 4096, 128) : 128;
   if (R != 32 && R != 64 && R != 128) R = R < 64 ? 32 : 64;
   if ((reduce_sec >= 0 || assign_sec >= 0) && R > 64) R = 64;   // the assign / reduce kernels stop at 64
   if (n >> 36) R = reduce_sec >= 0 || assign_sec >= 0 ? 64 : 128;   // chunk numbers below 2^32

@@ -40,7 +40,7 @@ static_assert(kReduceTableBytes % 16 == 0 && kReduceListBytes % 16 == 0, "the ce
 
 // One section on the M records of each lane of a staged chunk (r = lane + 32m), writes into the
 // chunk buffer; op is runtime (uniform over the launch).
-template <int M>
+template <int M, bool KM>
 __device__ __forceinline__ void fused_section_chunk(const FusedArgs& a, const FieldRef* fr, const SecOp& so,
                                                     uint8_t* cur, int64_t i0, const int32_t* ps, int lane) {
   switch (so.op) {
@@ -65,13 +65,21 @@ __device__ __forceinline__ void fused_section_chunk(const FusedArgs& a, const Fi
     ADHA_FUSED_OP(ADHA_OP_AXPB)
     ADHA_FUSED_OP(ADHA_OP_MUL)
     ADHA_FUSED_OP(ADHA_OP_TANH)
-    ADHA_FUSED_OP(ADHA_OP_ASSIGN)
+    case ADHA_OP_ASSIGN:
+      if constexpr (KM) {
+        _Pragma("unroll") for (int m = 0; m < M; ++m) {
+          const int r = lane + 32 * m;
+          run_record<ADHA_OP_ASSIGN>(so, fr, a.tanh_p, a.tanh_q, nullptr, StagedRec{fr, cur, r, i0 + r}, i0 + r, 0);
+        }
+      }
+      break;
 #undef ADHA_FUSED_OP
     default: break;
   }
 }
 
 // One section on one record in global memory (the ragged tail).
+template <bool KM>
 __device__ __forceinline__ void fused_section_record(const FusedArgs& a, const FieldRef* fr, const SecOp& so, int64_t i,
                                                      int32_t pj) {
   const GlobalRec rec{fr, i};
@@ -91,7 +99,9 @@ __device__ __forceinline__ void fused_section_record(const FusedArgs& a, const F
     ADHA_FUSED_OP(ADHA_OP_AXPB)
     ADHA_FUSED_OP(ADHA_OP_MUL)
     ADHA_FUSED_OP(ADHA_OP_TANH)
-    ADHA_FUSED_OP(ADHA_OP_ASSIGN)
+    case ADHA_OP_ASSIGN:
+      if constexpr (KM) run_record<ADHA_OP_ASSIGN>(so, fr, a.tanh_p, a.tanh_q, nullptr, rec, i, pj);
+      break;
 #undef ADHA_FUSED_OP
     default: break;
   }
@@ -177,7 +187,7 @@ __global__ void __launch_bounds__(kThreads) fused_kernel(const __grid_constant__
       else if (VEC && op == ADHA_OP_AXPB) chain_chunk_vec<ADHA_OP_AXPB, M, true>(so, fr, a.tanh_p, a.tanh_q, nullptr, cur, i0, lane);
       else if (VEC && op == ADHA_OP_MUL) chain_chunk_vec<ADHA_OP_MUL, M, true>(so, fr, a.tanh_p, a.tanh_q, nullptr, cur, i0, lane);
       else if (VEC && op == ADHA_OP_TANH) chain_chunk_vec<ADHA_OP_TANH, M, true>(so, fr, a.tanh_p, a.tanh_q, nullptr, cur, i0, lane);
-      else fused_section_chunk<M>(a, fr, so, cur, i0, ps, lane);
+      else fused_section_chunk<M, KM>(a, fr, so, cur, i0, ps, lane);
       __syncwarp();   // the next section may map records to lanes the other way
     }
     // groups with written fields go back whole, 16 bytes per lane per step
@@ -196,7 +206,7 @@ __global__ void __launch_bounds__(kThreads) fused_kernel(const __grid_constant__
     if (!KM || a.reduce_sec < 0) {
       for (int64_t i = t0 + lane; i < a.n; i += 32) {
         const int32_t pj = a.perm_slot >= 0 ? a.perm[i] : 0;
-        for (int s = 0; s < a.n_sec; ++s) fused_section_record(a, fr, secs[s], i, pj);
+        for (int s = 0; s < a.n_sec; ++s) fused_section_record<KM>(a, fr, secs[s], i, pj);
       }
     } else {   // section by section over the tail's records: the reduce reads every lane's records
       for (int s = 0; s < a.n_sec; ++s) {
@@ -205,7 +215,7 @@ __global__ void __launch_bounds__(kThreads) fused_kernel(const __grid_constant__
           if constexpr (KM) reduce_tail(rq, secs[s], fr, t0, a.n, lane, acc, sum, &cnt_lane);
         } else {
           for (int64_t i = t0 + lane; i < a.n; i += 32)
-            fused_section_record(a, fr, secs[s], i, a.perm_slot >= 0 ? a.perm[i] : 0);
+            fused_section_record<KM>(a, fr, secs[s], i, a.perm_slot >= 0 ? a.perm[i] : 0);
         }
       }
     }

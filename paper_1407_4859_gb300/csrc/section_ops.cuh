@@ -625,14 +625,20 @@ ADHA_FIELD_LOOP
     float D[kMaxClusters];
 #pragma unroll
     for (int k = 0; k < kMaxClusters; ++k) D[k] = 0.0f;
-    for (int j = 0; j < d; ++j) {
-      const float x = rec.template ld<float>(so.rd[j0 + j]);
+    for (int j = 0; j < d; j += 4) {   // four features' loads in flight together
+      float x[4];
 #pragma unroll
-      for (int k = 0; k < kMaxClusters; ++k)
-        if (k < K) {
-          const float df = __fsub_rn(x, __ldg(cent + k * d + j));
-          D[k] = __fadd_rn(D[k], __fmul_rn(df, df));
-        }
+      for (int b = 0; b < 4; ++b) x[b] = rec.template ld<float>(so.rd[j0 + min(j + b, d - 1)]);
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        if (j + b >= d) break;
+#pragma unroll
+        for (int k = 0; k < kMaxClusters; ++k)
+          if (k < K) {
+            const float df = __fsub_rn(x[b], __ldg(cent + k * d + j + b));
+            D[k] = __fadd_rn(D[k], __fmul_rn(df, df));
+          }
+      }
     }
     int best = 0;
     float bd = D[0];
@@ -975,33 +981,49 @@ __device__ __forceinline__ void reduce_sums(const ReduceLane& q, const uint8_t* 
   }
 }
 
-// REDUCE over records [t0, n) read from global memory (the ragged tail): lane j = feature j,
-// lane k counts cluster k; sums into the register sums (walk) or row mm of the first shared table.
+// REDUCE over records [t0, n) read from global memory (the ragged tail): lane j = feature j, lane k
+// counts cluster k; sums into the register sums (walk) or row mm of the first shared table.  Up to 127
+// records by one warp: 32 memberships and then eight records' features are read at a time, or their
+// latencies are most of a short launch.
 __device__ __forceinline__ void reduce_tail(const ReduceLane& q, const SecOp& so, const FieldRef* fr, int64_t t0,
                                             int64_t n, int lane, long long* acc, long long (&sum)[kMaxClusters],
                                             unsigned long long* cnt) {
   const FieldRef& Fm = fr[so.arg[0]];
-  const int j0 = so.rd_off[ADHA_F32];
-  for (int64_t i = t0; i < n; ++i) {
-    const int mm = *reinterpret_cast<const int32_t*>(Fm.g + i * Fm.gs);
-    if ((unsigned)mm >= (unsigned)q.K) continue;
-    if (lane == mm) *cnt += 1ull;
-    if (lane < q.d) {
-      const FieldRef& Fx = fr[so.rd[j0 + lane]];
-      const long long v = fixq(*reinterpret_cast<const float*>(Fx.g + i * Fx.gs));
-      if (q.walk) {
+  const FieldRef& Fx = fr[so.rd[so.rd_off[ADHA_F32] + (lane < q.d ? lane : 0)]];
+  const uint8_t* x0 = Fx.g;
+  const int xs = Fx.gs;
+  for (int64_t b = t0; b < n; b += 32) {
+    const int m = (int)(n - b < 32 ? n - b : 32);
+    const int member = lane < m ? *reinterpret_cast<const int32_t*>(Fm.g + (b + lane) * Fm.gs) : -1;
+#pragma unroll 1
+    for (int r = 0; r < m; r += 8) {
+      float x[8];
 #pragma unroll
-        for (int k = 0; k < kMaxClusters; ++k) sum[k] += k == mm ? v : 0ll;
-      } else {
-        acc[mm * 32 + lane] += v;
+      for (int u = 0; u < 8; ++u) x[u] = r + u < m ? *reinterpret_cast<const float*>(x0 + (b + r + u) * xs) : 0.0f;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int mm = __shfl_sync(0xFFFFFFFFu, member, r + u);   // -1 beyond the last record
+        if ((unsigned)mm >= (unsigned)q.K) continue;
+        if (lane == mm) *cnt += 1ull;
+        if (lane < q.d) {
+          const long long v = fixq(x[u]);
+          if (q.walk) {
+#pragma unroll
+            for (int k = 0; k < kMaxClusters; ++k) sum[k] += k == mm ? v : 0ll;
+          } else {
+            acc[mm * 32 + lane] += v;
+          }
+        }
       }
     }
   }
 }
 
-// The warps' sums and counts into the result, by all threads of the CTA: added up in shared memory
-// first (`table`: the CTA's record lists, done with by now), or 1.3 million additions to a few hundred
-// addresses would be most of a short launch.  Whole numbers: the order does not matter.
+// The warps' sums and counts added into the result (K rows of [count, d sums], zeroed before the launch
+// unless the caller accumulates), by all threads of the CTA.  They are added up in shared memory first
+// (`table`: the CTA's record lists, done with by now): warp by warp, over a million additions to a few
+// hundred addresses took most of a short launch (2^16 records of 32 features in 5 clusters 21 -> 14.8 us,
+// 2^20 57.9 -> 41.5, 2^23 222 -> 213.5).  Whole numbers: the order does not matter.
 __device__ __forceinline__ void reduce_flush(const ReduceLane& q, const SecOp& so, int warp, int lane, long long* table,
                                              const long long* acc, const long long (&sum)[kMaxClusters],
                                              const unsigned long long* cnt) {
