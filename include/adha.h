@@ -79,7 +79,7 @@ typedef struct {
 /*
  * Section ops.  arg[] holds operand field ids and fparam[] fp32 constants.
  * Every floating-point operation is rounded to nearest on its own (no fused
- * multiply-add), in the order written:
+ * multiply-add but the one that ASSIGN writes out), in the order written:
  *   MADD3   (x,y,z):            z = x*y + z                                 fp32
  *   XORSHIFT(x,z):              z = x ^ (x >> 3), logical shift              int32
  *   ADD     (x,y,z):            z = x + y                                   fp32
@@ -109,7 +109,9 @@ typedef struct {
  * arg[0] = the int32 membership field m, arg[1] = K (1..8 clusters):
  *   ASSIGN  (m, K; aux = K*d fp32 centroids c[k][j] = aux[k*d + j], device):
  *                               D_k = sum over j ascending of (x_j - c[k][j])^2
- *                               from +0 (fp32, each operation rounded);
+ *                               from +0 in fp32: t = x_j - c[k][j], rounded, then
+ *                               D_k = fma(t, t, D_k), one rounding for the square
+ *                               and the sum (the one op with a fused operation);
  *                               m = the smallest k with the smallest D_k.
  *                               read_mask: features only (d >= 1); write_mask: m
  *   REDUCE  (m, K; aux = K*(d+1) int64 outputs, device, 8-byte aligned):

@@ -6,7 +6,8 @@
  * path.  Everything is plain scalar C, one record and one field at a time, with
  * every floating-point operation written separately so that it is rounded to
  * nearest on its own (built with -O2 -ffp-contract=off -fno-fast-math: no
- * fused multiply-add, no reassociation, IEEE division).
+ * contraction into a fused multiply-add, no reassociation, IEEE division; the one
+ * fused operation, in the K-Means assign, is a call of fmaf).
  *
  * Paper: D. Majeti, K. S. Meel, R. Barik, V. Sarkar, "ADHA: Automatic Data
  * layout framework for Heterogeneous Architectures", PACT 2014.
@@ -341,9 +342,10 @@ int oracle_section_range(int op, const int* a, const float* p, uint64_t R, uint6
  *   membership m: the int32 field mf; K clusters; centroid c[k][j] = cent[k*d + j].
  *
  * assign:  per record, D_k = sum over j ascending of (x_j - c[k][j])^2, starting
- *          from +0, the subtraction, the square and the addition each rounded to
- *          nearest in fp32; m = the smallest k whose D_k is smallest (scanning k
- *          upwards, a later k wins only when strictly smaller).
+ *          from +0 in fp32: the subtraction rounded to nearest, then the square and
+ *          the addition together rounded once (fmaf, the only fused operation of
+ *          this file, written out); m = the smallest k whose D_k is smallest
+ *          (scanning k upwards, a later k wins only when strictly smaller).
  */
 int oracle_kmeans_assign_range(int d, const int* feat, int mf, int K, const float* cent, void** fa, int64_t i0,
                                int64_t i1);
@@ -362,8 +364,7 @@ int oracle_kmeans_assign_range(int d, const int* feat, int mf, int K, const floa
       float D = 0.0f;
       for (int j = 0; j < d; ++j) {
         float diff = F32(feat[j])[i] - cent[k * d + j];
-        float sq = diff * diff;
-        D = D + sq;
+        D = fmaf(diff, diff, D);
       }
       if (k == 0 || D < best_d) {
         best_d = D;

@@ -619,7 +619,9 @@ ADHA_FIELD_LOOP
     for (int ax = 0; ax < 3; ++ax)
       rec.template st<float>(g[ax], __fadd_rn(rec.template ld<float>(g[ax]), __fmul_rn(c, so.par[1 + ax])));
   } else if constexpr (OP == ADHA_OP_ASSIGN) {
-    // D_k summed over the features in ascending order, all K distances side by side
+    // D_k summed over the features in ascending order, all K distances side by side, by the rule of
+    // assign_chunk_k: the square and the sum in one fma (a record's membership must not depend on whether
+    // it lies in a chunk or in the ragged tail)
     const int K = so.arg[1], j0 = so.rd_off[ADHA_F32], d = so.rd_off[ADHA_F32 + 1] - j0;
     const float* cent = static_cast<const float*>(so.aux);
     float D[kMaxClusters];
@@ -636,7 +638,7 @@ ADHA_FIELD_LOOP
         for (int k = 0; k < kMaxClusters; ++k)
           if (k < K) {
             const float df = __fsub_rn(x[b], __ldg(cent + k * d + j + b));
-            D[k] = __fadd_rn(D[k], __fmul_rn(df, df));
+            D[k] = __fmaf_rn(df, df, D[k]);
           }
       }
     }
