@@ -919,6 +919,9 @@ static int plan_section(const Layout& L, void* const* ptrs, const adha_section* 
     for (int w = 0; w < 3; ++w)
       for (int k = 0; k < (s->op == ADHA_OP_DRIFT ? 6 : s->op == ADHA_OP_KICK ? 4 : 3); ++k)
         if (k != w && s->arg[k] == s->arg[w]) a.alias = 1;
+  // Records too wide for the chunk in shared memory: first shorter chunks, then no room after the staged
+  // records, then one chunk buffer (448-byte records do not fit twice, 416-byte ones only without the room).
+  bool room = true;
   for (;;) {
     a.n = n;
     a.R = R;
@@ -950,13 +953,14 @@ static int plan_section(const Layout& L, void* const* ptrs, const adha_section* 
       const bool wide = (L.stride[g] > 8 || a.alias) && written > 0;
       a.writeback[k] = (int8_t)(a.alias ? wide : wb_mode == 1 ? 0 : wb_mode == 2 ? wide : (wide && 4 * written >= L.stride[g]));
       a.n_writeback += a.writeback[k];
-      a.pad[k] = staged_room(L.stride[g]) ? 1 : 0;
+      a.pad[k] = room && staged_room(L.stride[g]) ? 1 : 0;
+      const int stride = L.stride[g] + 16 * a.pad[k];
       for (int f : L.groups[g]) {
         a.f[f].s0 = off + L.offset_of[f];
-        a.f[f].ss = staged_stride(L.stride[g]);
+        a.f[f].ss = stride;
         a.f[f].wsm = a.writeback[k];
       }
-      off += slice_bytes(R, staged_stride(L.stride[g]), walk);
+      off += slice_bytes(R, stride, walk);
     }
     if (s->op == ADHA_OP_GATHER) {
       a.perm_slot = a.n_load;
@@ -978,8 +982,16 @@ static int plan_section(const Layout& L, void* const* ptrs, const adha_section* 
       if ((has(staged, f) || has(s->write_mask, f)) && L.groups[L.group_of[f]].size() != 1) a.vec = 0;
     plan->smem = section_smem_bytes(a);
     if (plan->smem <= (size_t)kSmemLimit) break;
-    if (R <= 32) return fail(ADHA_EINVAL, "section records too wide for a 32-record chunk");
-    R /= 2;
+    if (R > 32) {
+      R /= 2;
+    } else if (room) {
+      room = false;
+    } else if (buffers == 2) {
+      buffers = 1;
+      room = true;
+    } else {
+      return fail(ADHA_EINVAL, "section records too wide for a 32-record chunk");
+    }
   }
   fill_secop_offsets(&a.s, a.f);
   tanh_coefficients(a.tanh_p, a.tanh_q);
@@ -1203,6 +1215,7 @@ static int plan_fused(const Layout& L, void* const* ptrs, const adha_section* s,
   if ((reduce_sec >= 0 || assign_sec >= 0) && R > 64) R = 64;   // the assign / reduce kernels stop at 64
   if (n >> 36) R = reduce_sec >= 0 || assign_sec >= 0 ? 64 : 128;   // chunk numbers below 2^32
   const bool walk = reduce_sec >= 0 && reduce_walks(L, &s[reduce_sec]);
+  int buffers = tuned_buffers == 1 || tuned_buffers == 2 ? tuned_buffers : kFusedBuffers;
   for (;;) {
     a.n = n;
     a.R = R;
@@ -1244,7 +1257,7 @@ static int plan_fused(const Layout& L, void* const* ptrs, const adha_section* s,
     }
     a.in_bytes = off;
     a.vec = vec ? 1 : 0;
-    a.buffers = tuned_buffers == 1 || tuned_buffers == 2 ? tuned_buffers : kFusedBuffers;
+    a.buffers = buffers;
     a.n_sec = m;
     a.reduce_sec = reduce_sec;
     a.assign_sec = assign_sec;
@@ -1252,8 +1265,9 @@ static int plan_fused(const Layout& L, void* const* ptrs, const adha_section* s,
     a.reduce_walk = walk ? 1 : 0;
     plan->smem = fused_smem_bytes(a);
     if (plan->smem <= (size_t)kSmemLimit) break;
-    if (R <= 32) return fail(ADHA_EINVAL, "the fused run's records are too wide for a 32-record chunk");
-    R /= 2;
+    if (R > 32) R /= 2;
+    else if (buffers == 2) buffers = 1;   // asked for two, which do not fit
+    else return fail(ADHA_EINVAL, "the fused run's records are too wide for a 32-record chunk");
   }
   a.n_sec = m;
   for (int k = 0; k < m; ++k) {
