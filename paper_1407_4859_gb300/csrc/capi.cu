@@ -846,6 +846,39 @@ static int check_section(const Layout& L, const adha_section* s, int64_t n, bool
   return 0;
 }
 
+// Whether a section stages structs of `stride` bytes with 16 bytes of room after each.  Without it 32 lanes'
+// words of one field lie on 32 / gcd(stride / 4, 32) banks: 8 lanes share one at 32 or 96 bytes, 16 at 64, 32 at
+// 128, with it 4.  The room takes shared memory (half as much again at 32 bytes), and with it warps, which the
+// sections that read few of a struct's fields need more.  us without -> with, 4000037 records:
+// * 128 bytes: mix of 32 fields 1351 -> 344, drift 173 -> 140, assign 220 -> 134, axpb 133 -> 130; always;
+// * 64: mix 372 -> 150, drift (6 accesses) 93 -> 75, kick (4) 82 -> 76, bin (3) 71 -> 74, axpb 68 -> 74;
+// * 32: mix 114 -> 79, drift (9) 63 -> 55, gather (6) 87 -> 83, ke (4) 31 -> 39, bin (3) 27 -> 36, tanh 38 -> 48;
+//   96: mix of 24 fields 329 -> 235, reading 24 and writing one 134 -> 124, axpb 99 -> 109; fp64 fields conflict
+//   half as often (32 bytes, mix of 4: 82 -> 91);
+// * assign reads four features at a time where they lie together (32 bytes 43 -> 46, 64: 87 -> 71, 96: 98 ->
+//   102; 32 bytes in another order 75 -> 70), and in reduce the lanes read one record's consecutive words, only the
+//   membership a column (four 32-byte structs 109 -> 114, 128: 109 -> 105).
+static bool section_room(const Layout& L, int g, const adha_section* s, uint64_t staged, bool writeback) {
+  const int stride = L.stride[g];
+  if (!staged_room(stride)) return false;
+  if (stride % 128 == 0) return true;
+  if (s->op == ADHA_OP_REDUCE) return false;
+  int halves = 0;   // accesses per record, two for each, one for an fp64 field at 32, 96, ... bytes
+  for (int f : L.groups[g])
+    halves += (has(staged, f) + (writeback && has(s->write_mask, f))) * (stride % 64 && dtype_size(L.dtype[f]) == 8 ? 1 : 2);
+  if (s->op == ADHA_OP_ASSIGN) {
+    std::vector<int> x;   // the features in order
+    for (int f = 0; f < L.F; ++f)
+      if (has(s->read_mask, f)) x.push_back(f);
+    for (size_t j = 0; j + 4 <= x.size(); j += 4) {
+      bool four = L.group_of[x[j]] == g && L.offset_of[x[j]] % 16 == 0;
+      for (int b = 1; b < 4 && four; ++b) four = L.group_of[x[j + b]] == g && L.offset_of[x[j + b]] == L.offset_of[x[j]] + 4 * b;
+      if (four) halves -= 6;
+    }
+  }
+  return stride % 64 == 0 ? halves >= 8 : 8 * halves >= 3 * stride;
+}
+
 int check_section_layout(const Layout& L, const adha_section* s, int64_t n) { return check_section(L, s, n, false); }
 
 struct SectionPlan {
@@ -921,7 +954,8 @@ static int plan_section(const Layout& L, void* const* ptrs, const adha_section* 
         if (k != w && s->arg[k] == s->arg[w]) a.alias = 1;
   // Records too wide for the chunk in shared memory: first shorter chunks, then no room after the staged
   // records, then one chunk buffer (448-byte records do not fit twice, 416-byte ones only without the room).
-  bool room = true;
+  // room: 2 where section_room says so, 1 for structs of a multiple of 64 bytes only, 0 none.
+  int room = 2;
   for (;;) {
     a.n = n;
     a.R = R;
@@ -938,7 +972,7 @@ static int plan_section(const Layout& L, void* const* ptrs, const adha_section* 
       a.f[f].wsm = 0;
       a.f[f].dtype = L.dtype[f];
     }
-    int off = 0;
+    int off = 0, odd_rooms = 0;
     a.n_writeback = 0;
     for (int k = 0; k < a.n_load; ++k) {
       const int g = groups[k];
@@ -953,7 +987,9 @@ static int plan_section(const Layout& L, void* const* ptrs, const adha_section* 
       const bool wide = (L.stride[g] > 8 || a.alias) && written > 0;
       a.writeback[k] = (int8_t)(a.alias ? wide : wb_mode == 1 ? 0 : wb_mode == 2 ? wide : (wide && 4 * written >= L.stride[g]));
       a.n_writeback += a.writeback[k];
-      a.pad[k] = room && staged_room(L.stride[g]) ? 1 : 0;
+      const bool odd = L.stride[g] % 64 != 0;
+      a.pad[k] = room > (odd ? 1 : 0) && section_room(L, g, s, staged, a.writeback[k]) ? 1 : 0;
+      if (odd) odd_rooms += a.pad[k];
       const int stride = L.stride[g] + 16 * a.pad[k];
       for (int f : L.groups[g]) {
         a.f[f].s0 = off + L.offset_of[f];
@@ -981,14 +1017,20 @@ static int plan_section(const Layout& L, void* const* ptrs, const adha_section* 
     for (int f = 0; f < L.F && a.vec; ++f)
       if ((has(staged, f) || has(s->write_mask, f)) && L.groups[L.group_of[f]].size() != 1) a.vec = 0;
     plan->smem = section_smem_bytes(a);
+    // not where it leaves an SM with one CTA instead of two (two 96-byte structs 663 -> 915 us)
+    const size_t odd_bytes = (size_t)kWarps * buffers * R * 16 * odd_rooms, two = kSmemPerSM / 2 - kSmemReservedPerCTA;
+    if (odd_rooms && plan->smem > two && plan->smem - odd_bytes <= two) {
+      room = 1;
+      continue;
+    }
     if (plan->smem <= (size_t)kSmemLimit) break;
     if (R > 32) {
       R /= 2;
     } else if (room) {
-      room = false;
+      room = 0;
     } else if (buffers == 2) {
       buffers = 1;
-      room = true;
+      room = 2;
     } else {
       return fail(ADHA_EINVAL, "section records too wide for a 32-record chunk");
     }
