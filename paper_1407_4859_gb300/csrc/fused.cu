@@ -35,7 +35,7 @@ __host__ __device__ constexpr int fused_table_bytes(int n_sec, int n_pieces) {
 
 // After the chunk buffers: a REDUCE's two sum tables per warp (unless it walks) and its record
 // lists (see reduce_chunk_any), then an ASSIGN's centroid table.
-static_assert(kReduceTableBytes % 16 == 0 && kReduceListBytes % 16 == 0, "the centroid table stays 16-byte aligned");
+static_assert(kReduceTableBytes % 16 == 0 && kReduceListBytes % 16 == 0 && kReduceFlushBytes % 16 == 0, "the centroid table stays 16-byte aligned");
 
 
 // One section on the M records of each lane of a staged chunk (r = lane + 32m), writes into the
@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(kThreads) fused_kernel(const __grid_constant__
       if (nb == 2) zero_records(a, R, buf1, lane);
     }
     idx = reinterpret_cast<int*>(extra) + warp * kReduceList;
-    extra += kReduceListBytes;
+    extra += a.reduce_walk ? kReduceListBytes : kReduceFlushBytes;
 #pragma unroll
     for (int k = 0; k < (KM ? kMaxClusters : 1); ++k) sum[k] = 0;
   }
@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(kThreads) fused_kernel(const __grid_constant__
 
 size_t fused_smem_bytes(const FusedArgs& a) {
   return fused_table_bytes(a.n_sec, stage_pieces(a, a.R)) + (size_t)kWarps * a.buffers * a.in_bytes +
-         (a.reduce_sec >= 0 ? (a.reduce_walk ? 0 : kReduceTableBytes) + kReduceListBytes : 0) +
+         (a.reduce_sec >= 0 ? reduce_smem_bytes(a.reduce_walk != 0) : 0) +
          (a.assign_sec >= 0 ? (size_t)kCentroidBytes : 0);
 }
 

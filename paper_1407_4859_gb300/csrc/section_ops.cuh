@@ -838,11 +838,18 @@ struct ReduceLane {
   bool walk;              // sum cluster by cluster into registers (see reduce_chunk_any)
 };
 
-// Shared memory of a REDUCE per CTA: the two sum tables of every warp (when it does not walk) and
-// every warp's record list.
+// Shared memory of a REDUCE per CTA: every warp's record list (walk), or the two sum tables of every warp;
+// and the table of reduce_flush, in the lists' place or after the tables.  (Lists that are not used left an
+// SM with one CTA instead of two: 4000037 records of 32 features in 13 groups, one-field ones among them,
+// 237 us, 170 without.)
 constexpr size_t kReduceTableBytes = (size_t)kWarps * 2 * (kMaxClusters + 1) * 32 * 8;
 constexpr int kReduceList = 128 + 4 * kMaxClusters + 8;   // 128 records, clusters in whole fours, 8 to read ahead
 constexpr size_t kReduceListBytes = (size_t)kWarps * kReduceList * 4;
+constexpr size_t kReduceFlushBytes = (size_t)kMaxClusters * (kMaxReduceFeatures + 1) * 8;
+static_assert(kReduceListBytes >= kReduceFlushBytes, "the flush table fits the record lists");
+__host__ __device__ constexpr size_t reduce_smem_bytes(bool walk) {
+  return walk ? kReduceListBytes : kReduceTableBytes + kReduceFlushBytes;
+}
 
 // walk: every feature lies in a slice wider than one field (decided on the host, which sizes the
 // shared tables only for the other way).
@@ -1023,13 +1030,12 @@ __device__ __forceinline__ void reduce_tail(const ReduceLane& q, const SecOp& so
 
 // The warps' sums and counts added into the result (K rows of [count, d sums], zeroed before the launch
 // unless the caller accumulates), by all threads of the CTA.  They are added up in shared memory first
-// (`table`: the CTA's record lists, done with by now): warp by warp, over a million additions to a few
+// (`table`: see reduce_smem_bytes; the record lists are done with by now): warp by warp, over a million additions to a few
 // hundred addresses took most of a short launch (2^16 records of 32 features in 5 clusters 21 -> 14.8 us,
 // 2^20 57.9 -> 41.5, 2^23 222 -> 213.5).  Whole numbers: the order does not matter.
 __device__ __forceinline__ void reduce_flush(const ReduceLane& q, const SecOp& so, int warp, int lane, long long* table,
                                              const long long* acc, const long long (&sum)[kMaxClusters],
                                              const unsigned long long* cnt) {
-  static_assert(kReduceListBytes >= kMaxClusters * 33 * 8, "the table fits the record lists");
   const int d = q.d, row = d + 1;
   for (int w = 0; w < kWarps; ++w) {
     __syncthreads();

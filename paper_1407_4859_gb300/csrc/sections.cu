@@ -34,7 +34,7 @@ __global__ void __launch_bounds__(kThreads) section_kernel(const __grid_constant
   uint8_t* buf1 = buf0 + (nb - 1) * a.in_bytes;
   uint8_t* extra = bufs + (size_t)kWarps * nb * a.in_bytes;
   // REDUCE: counts and (walk) sums in registers; after the chunk buffers the warp's two sum
-  // tables (not walk) and its record list (walk)
+  // tables (not walk) or its record list (walk), see reduce_smem_bytes
   long long* acc = nullptr;
   int* idx = nullptr;
   unsigned long long cnt = 0;   // REDUCE: lane k counts cluster k
@@ -221,8 +221,7 @@ __global__ void __launch_bounds__(kThreads) backward_kernel(const __grid_constan
 }
 
 size_t section_smem_bytes(const SectionArgs& a) {
-  // REDUCE: two (K+1) x 32 int64 tables per warp unless it walks, and a record list per warp
-  const size_t acc = a.s.op == ADHA_OP_REDUCE ? (a.reduce_walk ? 0 : kReduceTableBytes) + kReduceListBytes : 0;
+  const size_t acc = a.s.op == ADHA_OP_REDUCE ? reduce_smem_bytes(a.reduce_walk != 0) : 0;
   const size_t cent = a.s.op == ADHA_OP_ASSIGN ? (size_t)kCentroidBytes : 0;
   return (size_t)stage_pieces(a, a.R) * sizeof(StagePiece) + (size_t)kWarps * a.buffers * a.in_bytes + acc + cent;
 }
