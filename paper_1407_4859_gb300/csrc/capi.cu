@@ -916,10 +916,20 @@ static int plan_section(const Layout& L, void* const* ptrs, const adha_section* 
   for (int g : groups) rec += L.stride[g];
   if (s->op == ADHA_OP_GATHER) rec += 4;
   const bool walk = reduce_walks(L, s);
+  // assign on narrow records, enough of them for long chunks: one wave of long chunks in two buffers, there is
+  // little to compute per chunk.  us, (64 records, one buffer, 8 waves) -> so: 4000037 records of 12 bytes 27.4 ->
+  // 17.5, of 28 (one array per field) 45.6 -> 37.8, 1500007 of 20 14.6 -> 12.8, but of 28 15.5 -> 17.2, 300007 of 20
+  // 7.2 -> 8.2 and 8388608 of 32 99 -> 115.
+  int sms = 0;
+  if (int rc = sm_count(&sms)) return rc;
+  const bool narrow = s->op == ADHA_OP_ASSIGN && !tuned_R && !buffers && rec <= 28 &&
+                      n >= (int64_t)128 * sms * (rec <= 20 ? 32 : 128);
   int R = 128;
   if (tuned_R) {
     R = std::max(32, std::min(tuned_R, 128));
     if (R != 32 && R != 64 && R != 128) R = R < 64 ? 32 : 64;   // 96 -> 64: the kernels exist for 32, 64, 128
+  } else if (narrow) {
+    buffers = 2;
   } else if (s->op == ADHA_OP_ASSIGN || walk) {
     // long compute per chunk: two or more records per lane share the operand loads, one buffer makes
     // room for 16 warps.  8388608 x 132 bytes, (records per chunk, buffers): assign (32,2) 332 us,
@@ -938,10 +948,10 @@ static int plan_section(const Layout& L, void* const* ptrs, const adha_section* 
   if (!tuned_R) {
     // few records: shorter chunks, so that every SM's schedulers have a warp; a reduce takes its chunk's
     // records one after another, and gains from 24 chunks per SM (151651 records of 12 bytes 20.9 -> 13.3
-    // us, 343024 of 56 bytes 31.6 -> 21.4)
-    int sms = 0;
-    if (int rc = sm_count(&sms)) return rc;
-    while (R > 32 && n < (int64_t)R * sms * (s->op == ADHA_OP_REDUCE ? 24 : 4)) R /= 2;
+    // us, 343024 of 56 bytes 31.6 -> 21.4), an assign on wide records from 40 (300007 records of 128 bytes 21.5 ->
+    // 19.4, of 33 arrays 28.2 -> 21.7; 1500007 of 33 arrays 60.8 -> 61.4)
+    const int chunks = s->op == ADHA_OP_REDUCE ? 24 : s->op == ADHA_OP_ASSIGN && rec > 28 ? 40 : 4;
+    while (R > 32 && n < (int64_t)R * sms * chunks) R /= 2;
   }
   if (buffers != 1) buffers = 2;
   if (n >> 36) R = 128;   // chunk numbers below 2^32 (so many records are a few bytes each: 128 of them fit)
@@ -1042,9 +1052,8 @@ static int plan_section(const Layout& L, void* const* ptrs, const adha_section* 
   int blocks = 0;
   if (int rc = cached_occupancy(1000 + 1000 * s->op + a.R + a.vec, plan->smem, &blocks)) return rc;
   // assign has little to set up per CTA and its stores are uneven work: 280 us in one wave, 262 at 8
-  int waves = 1, sms = 0;
-  if (int rc = sm_count(&sms)) return rc;
-  if (s->op == ADHA_OP_ASSIGN) waves = waves_for(a.n_chunks, sms, blocks * kWarps, 8, 2);
+  int waves = 1;
+  if (s->op == ADHA_OP_ASSIGN && !narrow) waves = waves_for(a.n_chunks, sms, blocks * kWarps, 8, 2);
   return finish_grid(a.n_chunks, blocks * waves, &plan->grid);
 }
 
