@@ -1351,6 +1351,10 @@ static int plan_fused(const Layout& L, void* const* ptrs, const adha_section* s,
   }
   const int M = R / 32;
   if (int rc = cached_occupancy(200 + 10 * M + a.vec + 2 * (fused_is_km(a) ? 1 : 0), plan->smem, &blocks)) return rc;
+  // structs: 32 warps per SM stream better than 64.  4000037 records, us at all the registers allow / 5 / 4 CTAs: nine
+  // stress sections in 80-byte structs 841 / 807 / 824, 300007 of them 79 / 81 / 73; three sections on 24-byte structs
+  // 53.6 / 51.5 / 50.4, four on 56-byte ones 113.8 / 113.8 / 110.4.  One-field groups 1.00
+  if (!a.vec && !fused_is_km(a)) blocks = std::min(blocks, 4);
   return finish_grid(a.n_chunks, blocks, &plan->grid);
 }
 
