@@ -378,8 +378,12 @@ __global__ void __launch_bounds__(kChainThreads) chain_backward_kernel(const __g
     for (int k = 0; k < a.n_copy; ++k) {
       const ChainCopy& cp = a.copy[k];
       const int64_t b0 = i0 * cp.stride;
-      const int bytes = (int)((whole ? (int64_t)R : a.n - i0) * cp.stride);
-      for (int p = lane * 4; p < bytes; p += 128)
+      const int bytes = (int)((whole ? (int64_t)R : a.n - i0) * cp.stride), whole16 = bytes / 16 * 16;
+      // (R * 4 bytes is a multiple of 16: every chunk starts on one)
+#pragma unroll 4
+      for (int p = lane * 16; p < whole16; p += 512)
+        *reinterpret_cast<uint4*>(cp.dst + b0 + p) = *reinterpret_cast<const uint4*>(cp.src + b0 + p);
+      for (int p = whole16 + lane * 4; p < bytes; p += 128)
         *reinterpret_cast<float*>(cp.dst + b0 + p) = *reinterpret_cast<const float*>(cp.src + b0 + p);
     }
     __syncwarp();
