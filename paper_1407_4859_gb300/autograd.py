@@ -138,7 +138,7 @@ class SegmentFn(torch.autograd.Function):
              for k, x in enumerate(grads)]
         # the incoming gradients stay as they are: the last run's pass writes buffers of its own,
         # which the earlier runs then update in place
-        out = [torch.empty_like(x) for x in g]
+        out = [torch.empty_like(x) for x in g] if ctx.runs else _copy(schema, n, layout, g)
         for secs, saved in reversed(ctx.runs):
             adha_chain_backward(schema, n, layout, ctx.state, g, out, secs, saved)
             g = out
