@@ -10,20 +10,23 @@ fp32, so a group's struct is k contiguous floats).  Three autograd Functions:
 * SegmentFn: runs a run of axpb / mul / tanh sections in place in one layout, as chain runs
   (adha_chain_forward) that save what the written fields held before the run; its backward
   (adha_chain_backward) puts that back, runs the sections again on chip and walks them in reverse,
-  propagating the adjoints.
+  propagating the adjoints.  A few sections on wide structs run one by one instead, each saving the
+  value it overwrites, and its adjoint kernel (adha_section_backward) restores it.  (A schema with other
+  types than fp32 runs forward that way too; there is no backward for it.)
 * CopyFn: a copy of the state by the remap kernel, where the first section keeps the input layout.
 
 DifferentiableProgram strings them together for a whole program under a layout plan.  Every
 forward and backward step runs in the library's kernels; PyTorch only allocates and orders them.
-Memory: the forward keeps one saved field (n floats) per written field of each run and every layout's
-moved groups;
+Memory: the forward keeps one saved field (n floats) per written field of each chain run, or per section run
+on its own, and every layout's moved groups;
 the backward hands the program's state back to what it was before each segment, in place, so the
 forward outputs hold the input-side values once backward() has run (copy them first if needed).
 """
 import torch
 
 from ._lib import adha_section
-from .api import adha_chain_backward, adha_chain_forward, adha_chain_plan, adha_remap, adha_run_section, c_section
+from .api import (adha_chain_backward, adha_chain_forward, adha_chain_plan, adha_remap, adha_run_section,
+                  adha_section_backward, c_section)
 
 
 def _copy(schema, n, layout, groups):
@@ -103,17 +106,44 @@ class RemapFn(torch.autograd.Function):
         return (None,) + tuple(gs[s] for s in moved_s)
 
 
+def _faster_one_by_one(n, layout, sections):
+    """Whether a short segment on structs runs section by section: a chain run moves whole structs, a record
+    per lane, however few of their fields it touches.  Modelled ns per record, from runs of 2^22 records: a
+    chain run 0.0018 per byte of the structs it touches (0.0024 from 128 bytes on, 0.0037 where the size is
+    no multiple of 16) and a copy of the other gradients, sections 0.022 per operand in a struct and 0.0005 per
+    byte of the structs they read, and a copy of all gradients.  Forward + backward of 64 fields in one struct, chain run / one by one: 1 section 2886 / 1342 us,
+    2 2882 / 2104, 3 2879 / 2783, 8 2800 / 5500; 63 fields, 1 section 4235 / 1294, 4 4280 / 3020; 24 fields, 1
+    section 763 / 582, 2 780 / 800.  Where the difference is below 0.05 ms the launches cost more."""
+    copied = 8 * 1.55e-4   # a gradient's bytes, read and written, at the copy rate
+    structs = [g for g in layout.groups if len(g) > 1]
+    cost = [4 * len(g) * (0.0037 if len(g) % 4 else 0.0018 if len(g) < 32 else 0.0024) for g in structs]
+    single = copied * sum(map(len, layout.groups))
+    if n * (sum(cost) - single - 0.022 * len(sections)) <= 5e4:   # at most this, without a look at the operands
+        return False
+    at = {f: k for k, g in enumerate(structs) for f in g}
+    run = set()
+    for s in sections:
+        operands = [at[f] for f in s.args if f in at]
+        run.update(operands)
+        single += 0.022 * len(operands) + 0.0005 * sum(4 * len(structs[k]) for k in set(operands))
+    whole = sum(cost[k] if k in run else copied * len(structs[k]) for k in range(len(structs)))
+    return n * (whole - single) > 5e4
+
+
 class SegmentFn(torch.autograd.Function):
     @staticmethod
     def forward(ctx, meta, *groups):
         schema, n, layout, sections = meta
         runs = []
         k = 0
-        if any(schema.dtypes):   # other types than fp32 (forward only): chain runs do not take them
+        # other types than fp32 (forward only): chain runs do not take them
+        ctx.one_by_one = any(schema.dtypes) or _faster_one_by_one(n, layout, sections)
+        if ctx.one_by_one:
             for s in sections:
+                cs = c_section(s)
                 save = torch.empty(n, dtype=torch.float32, device="cuda")
-                adha_run_section(schema, n, layout, groups, c_section(s), save=save)
-                runs.append(((adha_section * 1)(c_section(s)), save))
+                adha_run_section(schema, n, layout, groups, cs, save=save)
+                runs.append((cs, save))
             k = len(sections)
         while k < len(sections):
             secs = (adha_section * (len(sections) - k))(*[c_section(s) for s in sections[k:]])
@@ -136,12 +166,17 @@ class SegmentFn(torch.autograd.Function):
         g = [x.contiguous() if x is not None else torch.zeros((n, len(layout.groups[k])), dtype=torch.float32,
                                                               device="cuda")
              for k, x in enumerate(grads)]
-        # the incoming gradients stay as they are: the last run's pass writes buffers of its own,
-        # which the earlier runs then update in place
-        out = [torch.empty_like(x) for x in g] if ctx.runs else _copy(schema, n, layout, g)
-        for secs, saved in reversed(ctx.runs):
-            adha_chain_backward(schema, n, layout, ctx.state, g, out, secs, saved)
-            g = out
+        # the incoming gradients stay as they are: the last run's pass writes buffers of its own (the adjoint
+        # kernel works in place, on copies), which the earlier ones then update in place
+        if ctx.one_by_one or not ctx.runs:
+            out = _copy(schema, n, layout, g)
+            for cs, save in reversed(ctx.runs):
+                adha_section_backward(schema, n, layout, ctx.state, out, cs, save)
+        else:
+            out = [torch.empty_like(x) for x in g]
+            for secs, saved in reversed(ctx.runs):
+                adha_chain_backward(schema, n, layout, ctx.state, g, out, secs, saved)
+                g = out
         # the state tensors' grad_fn refers to ctx: drop them here, or the step's memory waits for
         # Python's cycle collector
         ctx.runs = None
