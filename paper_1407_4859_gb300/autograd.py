@@ -110,15 +110,16 @@ def _faster_one_by_one(n, layout, sections):
     """Whether a short segment on structs runs section by section: a chain run moves whole structs, a record
     per lane, however few of their fields it touches.  Modelled ns per record, from runs of 2^22 records: a
     chain run 0.0018 per byte of the structs it touches (0.0024 from 128 bytes on, 0.0037 where the size is
-    no multiple of 16) and a copy of the other gradients, sections 0.022 per operand in a struct and 0.0005 per
-    byte of the structs they read, and a copy of all gradients.  Forward + backward of 64 fields in one struct, chain run / one by one: 1 section 2886 / 1342 us,
-    2 2882 / 2104, 3 2879 / 2783, 8 2800 / 5500; 63 fields, 1 section 4235 / 1294, 4 4280 / 3020; 24 fields, 1
-    section 763 / 582, 2 780 / 800.  Where the difference is below 0.05 ms the launches cost more."""
+    no multiple of 16) and a copy of the other gradients; sections 0.022 per operand in a struct, 0.0005 per
+    byte of the structs they read, and a copy of all gradients; and 0.03 ms of the host for a section's
+    launches.  Forward + backward, chain run / one by one: 64 fields in a struct, 1 section 2886 / 1342 us, 2
+    2882 / 2104, 3 2879 / 2783; 63 fields 1 section 4235 / 1294, 4 4280 / 3020; 24 fields 1 section 763 / 582."""
     copied = 8 * 1.55e-4   # a gradient's bytes, read and written, at the copy rate
     structs = [g for g in layout.groups if len(g) > 1]
     cost = [4 * len(g) * (0.0037 if len(g) % 4 else 0.0018 if len(g) < 32 else 0.0024) for g in structs]
     single = copied * sum(map(len, layout.groups))
-    if n * (sum(cost) - single - 0.022 * len(sections)) <= 5e4:   # at most this, without a look at the operands
+    launches = 3e4 * (2 + len(sections))
+    if n * (sum(cost) - single - 0.022 * len(sections)) <= launches:   # at most this, without a look at the operands
         return False
     at = {f: k for k, g in enumerate(structs) for f in g}
     run = set()
@@ -127,7 +128,7 @@ def _faster_one_by_one(n, layout, sections):
         run.update(operands)
         single += 0.022 * len(operands) + 0.0005 * sum(4 * len(structs[k]) for k in set(operands))
     whole = sum(cost[k] if k in run else copied * len(structs[k]) for k in range(len(structs)))
-    return n * (whole - single) > 5e4
+    return n * (whole - single) > launches
 
 
 class SegmentFn(torch.autograd.Function):
