@@ -602,6 +602,58 @@ static int plan_remap(const Layout& S, const void* const* src_ptrs, const Layout
   return finish_grid(a.n_chunks, blocks, &plan->grid);
 }
 
+// What a remap's launch shape goes by: the groups' widths on both sides and how much there is to move.
+struct RemapWidths {
+  int total = 0;            // staged bytes per record on both sides (without one-field destination groups)
+  double mb = 0;            // megabytes of source records
+  bool arrays = true;       // every source group holds one field
+  bool from_structs = true, into_structs = true;   // every source (built destination) group holds two or more
+  bool halves = false;      // a 16-bit field is moved
+  bool eights = true;       // every source struct's size is a multiple of 8
+  bool aligned = false;     // a built struct's size is a multiple of 64
+};
+
+static RemapWidths remap_widths(const Layout& S, const Layout& D, int64_t n, const std::vector<int>& build,
+                                const std::vector<int>& need, int in_rec, int out_rec) {
+  RemapWidths w;
+  w.total = in_rec + out_rec;
+  w.mb = 1e-6 * (double)n * in_rec;
+  for (int j : need) {
+    const bool one = S.groups[j].size() == 1;
+    w.arrays = w.arrays && one;
+    w.from_structs = w.from_structs && !one;
+    w.eights = w.eights && S.stride[j] % 8 == 0;
+  }
+  for (int d : build) {
+    w.into_structs = w.into_structs && D.groups[d].size() > 1;
+    w.aligned = w.aligned || D.stride[d] % 64 == 0;
+    for (int f : D.groups[d]) w.halves = w.halves || dtype_size(D.dtype[f]) == 2;
+  }
+  return w;
+}
+
+// Pairs of layouts that the schedule moves faster, once there is enough to move to pay for its set-up (a table per
+// CTA: 20 MB of records take 1.1 to 3 times as long by it as by columns).  Fitted to the times of 700 pairs at 20 to
+// 1000 MB of records; by columns / by schedule:
+// * structs into structs: above 448 staged bytes few warps are resident (150 MB 1.08 - 1.3, 400 MB 1.03 - 1.5; out of
+//   one struct, in one wave, 0.8 - 1.16, and above 864, 16 records per chunk, 1.1 - 1.8), and at 160 to 300 bytes where
+//   the sources' sizes are multiples of 8, whose words share banks (3 x 32 bytes into 96: 150 MB 1.26, 1000 1.23; 4 x
+//   12 into 48 0.94);
+// * arrays into structs: above 448 staged bytes 1.1 - 1.5, but 0.6 - 0.8 into structs of 128, 192 or 256 bytes,
+//   whose fields share banks in the schedule's buffer; 16-bit fields into structs of up to 16 bytes, where a row of
+//   32 records is 64 bytes (400 MB 0.97 - 1.85, mean 1.15);
+// * structs of at most 4 (8) bytes into arrays 1.6 (1.04 - 1.14).
+static bool schedule_faster(const RemapWidths& w, size_t sources, int out_rec) {
+  if (out_rec == 0) return (w.total <= 4 && w.mb >= 30) || (w.total <= 6 && w.mb >= 140) || (w.total <= 8 && w.mb >= 250);
+  if (w.arrays)
+    return (w.total > 448 && (w.total > 600 || !w.aligned) && w.mb >= 80) ||
+           (w.total <= 16 && w.mb >= 140) || (w.halves && w.total <= 32 && w.mb >= 200);
+  if (w.total > 864) return w.mb >= 40;
+  if (sources == 1) return false;
+  if (w.total > 448) return w.mb >= 120;
+  return w.from_structs && w.eights && !w.halves && w.total > 160 && w.total <= 300 && w.mb >= 120;
+}
+
 // The remap by columns of an untuned pair of layouts.  *fits = false (nothing planned) where plan_remap's
 // kernel is the better one or the records are too wide for the buffers here.
 static int plan_columns(const Layout& S, const void* const* src_ptrs, const Layout& D, void* const* dst_ptrs, int64_t n,
@@ -626,26 +678,40 @@ static int plan_columns(const Layout& S, const void* const* src_ptrs, const Layo
   // Records per chunk and waves of CTAs.  One buffer per warp.  A CTA has little to set up, and CTAs handed
   // out as others finish even out the SMs' different distances from memory (80-byte structs to one
   // array per field, us per 1 GB moved: 169 with one wave, 160 with 4, 154 with 16), except where
-  // every chunk gathers many slices.  By the schedule -> by columns, us per 1 GB:
+  // every chunk gathers many slices.  The limits below are a fit to sweeps of layouts, not a bound of the
+  // hardware; by the schedule -> by columns, us per 1 GB:
   // * structs to one array per field: 80 bytes 181 -> 154, 24 bytes 175 -> 151, 132 bytes 180 -> 154;
-  // * narrow records (both sides' buffers of 64 or more records leave 16 warps per SM) into several
-  //   structs or back: 36 bytes 171 -> 149, back 172 -> 152, 56 bytes 166 -> 157, back 167 -> 162;
-  // * wide records, 64 records while they leave 8 warps: one array per field into structs, one wave:
-  //   80 bytes 183 -> 158, 96 bytes 185 -> 172, 110 bytes of mixed types 219 -> 181, 132 bytes 183 in
-  //   both; structs into several structs, 8 waves: 92 bytes 249 -> 198, 116 bytes 205 -> 204.
-  const int total = in_rec + out_rec;
-  const bool several = need.size() > 2;
+  // * narrow records with one-field groups on a side (up to 112 staged bytes, 8 sources): 36 bytes into several
+  //   structs 171 -> 149, back 172 -> 152, 56 bytes 166 -> 157, back 167 -> 162;
+  // * wider ones, 64 records up to 220 staged bytes with several sources (140 with one or two): one array per
+  //   field into structs, one wave: 80 bytes 183 -> 158, 96 bytes 185 -> 172, 110 bytes of mixed types 219 -> 181,
+  //   132 bytes 183 in both; a struct into structs and arrays, 8 waves: 92 bytes 249 -> 198, 116 bytes 205 -> 204;
+  // * structs on both sides, and wide ones into anything: one wave below 600 MB of records without 16-bit fields
+  //   (8 waves / 1, us by columns: 150 MB in six 16-byte structs into 96 85 / 80, out of them 87 / 77, 256 bytes into
+  //   4 x 64 76 / 64; 1000 MB 1.02, with 16-bit fields 0.9 - 1.1); structs of 150 bytes or more into structs and arrays
+  //   too (150 MB 1.08 of the schedule's time / 0.91, 400 MB 1.05 / 0.94).
+  const RemapWidths w = remap_widths(S, D, n, build, need, in_rec, out_rec);
+  if (schedule_faster(w, need.size(), out_rec)) return 0;
+  const int total = w.total;
+  const bool several = need.size() > 2, one_wave = w.mb < 600 && total > 64 && !w.halves;
   bool table = false;   // the sources come in through the piece table
   int R, waves;
   if (out_rec == 0) {
     R = total <= 96 ? 128 : 64;
     waves = 16;
+  } else if (one_wave && need.size() == 1 && w.into_structs) {
+    R = total <= 224 ? 64 : 32;
+    waves = total <= 96 ? 4 : 1;
+  } else if (one_wave && w.from_structs && need.size() > 1) {
+    R = total <= 160 ? 64 : 32;
+    waves = 1;
+    table = need.size() > 4;
   } else if (total <= 112 && need.size() <= 8) {
     R = total <= 80 ? 128 : 64;
     waves = need.size() == 1 ? 16 : 8;
   } else {
     R = total <= (several ? 220 : 140) ? 64 : 32;
-    waves = several ? 1 : 8;
+    waves = several || (w.mb < 600 && need.size() == 1 && total > 300) ? 1 : 8;
     table = several;
   }
   auto warp_bytes = [&](int r) { return r * (in_rec + out_rec); };
