@@ -87,8 +87,11 @@ def _ptrs(bufs):
 
 def _stream_ptr(stream):
     if stream is None:
-        if torch.cuda.is_initialized():   # the current stream's handle without a Stream object around it
-            return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()))
+        # the current stream's handle without a Stream object around it (2 us of a launch), where this torch has
+        # the call: it is no public one
+        raw, device = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+        if raw and device and torch.cuda.is_initialized():
+            return ctypes.c_void_p(raw(device()))
         stream = torch.cuda.current_stream()
     return ctypes.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
 
