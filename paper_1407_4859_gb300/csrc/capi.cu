@@ -1560,7 +1560,8 @@ static uint64_t chain_read(const adha_section* s, int m) {
 }
 
 // Leading sections of s[0..m) that fit one run: at most kMaxChain, and at most kMaxChainExtra slots
-// beyond the fields' own (with the rows of 64 fields and their gradients, eight warps per SM).
+// beyond the fields' own (with the rows of 64 fields, their gradients and the span lists about 33 KB of shared memory
+// for 32 records: six warps per SM).
 static int chain_window(int F, const adha_section* s, int m) {
   int k = std::min(m, kMaxChain);
   while (k > 1 && chain_slots(F, chain_written(s, k) | chain_read(s, k), s, k).extra > kMaxChainExtra) k = std::max(1, k - 8);

@@ -54,49 +54,37 @@ __host__ __device__ __forceinline__ int chain_tables(const ChainArgs& a) {
   return n * (int)sizeof(ChainSpan);
 }
 
-// M floats of a lane as packed pairs (M = 1: the upper half is zero).
+// A lane's M floats, 1 or 2, as a packed pair (M = 1: the upper half is zero).
 template <int M>
-struct LaneVec {
-  static constexpr int H = (M + 1) / 2;
-  unsigned long long p[H];
-  __device__ __forceinline__ void load(const uint8_t* q) {
-    if constexpr (M == 2) {
-      p[0] = *reinterpret_cast<const unsigned long long*>(q);
-    } else {
-      p[0] = f2_pack(*reinterpret_cast<const float*>(q), 0.0f);
-    }
+__device__ __forceinline__ unsigned long long lane_load(const uint8_t* q) {
+  if constexpr (M == 2) return *reinterpret_cast<const unsigned long long*>(q);
+  return f2_pack(*reinterpret_cast<const float*>(q), 0.0f);
+}
+template <int M>
+__device__ __forceinline__ void lane_store(uint8_t* q, unsigned long long v) {
+  if constexpr (M == 2) {
+    *reinterpret_cast<unsigned long long*>(q) = v;
+  } else {
+    float lo, hi;
+    f2_unpack(v, &lo, &hi);
+    *reinterpret_cast<float*>(q) = lo;
   }
-  __device__ __forceinline__ void store(uint8_t* q) const {
-    if constexpr (M == 2) {
-      *reinterpret_cast<unsigned long long*>(q) = p[0];
-    } else {
-      float lo, hi;
-      f2_unpack(p[0], &lo, &hi);
-      *reinterpret_cast<float*>(q) = lo;
-    }
-  }
-};
+}
 
 // One section on the lane's records (`s`: the lane's first record of row 0).
 template <int M>
 __device__ __forceinline__ void chain_section(const ChainSec& c, uint8_t* s, const unsigned long long* P,
                                               const unsigned long long* Q, unsigned long long nz) {
-  constexpr int H = LaneVec<M>::H;
-  LaneVec<M> x, v;
-  x.load(s + c.x);
+  const unsigned long long x = lane_load<M>(s + c.x);
+  unsigned long long v;
   if (c.op == ADHA_OP_AXPB) {
-#pragma unroll
-    for (int h = 0; h < H; ++h) v.p[h] = f2_add_rn(f2_mul_alone(f2_pack(c.a, c.a), x.p[h], nz), f2_pack(c.b, c.b));
+    v = f2_add_rn(f2_mul_alone(f2_pack(c.a, c.a), x, nz), f2_pack(c.b, c.b));
   } else if (c.op == ADHA_OP_MUL) {
-    LaneVec<M> y;
-    y.load(s + c.y);
-#pragma unroll
-    for (int h = 0; h < H; ++h) v.p[h] = f2_mul_alone(x.p[h], y.p[h], nz);
+    v = f2_mul_alone(x, lane_load<M>(s + c.y), nz);
   } else {
-#pragma unroll
-    for (int h = 0; h < H; ++h) v.p[h] = tanh_pair(x.p[h], P, Q, nz);
+    v = tanh_pair(x, P, Q, nz);
   }
-  v.store(s + c.z);
+  lane_store<M>(s + c.z, v);
 }
 
 // The adjoint of one section (adha_section_backward's rule, in its order): gz = g[z], g[z] = 0, then
@@ -104,34 +92,21 @@ __device__ __forceinline__ void chain_section(const ChainSec& c, uint8_t* s, con
 // has them read from the row of zeros; zero_rows says which are left so.
 template <int M>
 __device__ __forceinline__ void chain_adjoint(const ChainAdj& c, const uint8_t* s, uint8_t* g, unsigned long long nz) {
-  constexpr int H = LaneVec<M>::H;
-  LaneVec<M> gz, gx;
-  gz.load(g + c.gz);
-  gx.load(g + c.gx_in);
+  const unsigned long long gz = lane_load<M>(g + c.gz);
+  unsigned long long gx = lane_load<M>(g + c.gx_in);
   if (c.op == ADHA_OP_AXPB) {
-#pragma unroll
-    for (int h = 0; h < H; ++h) gx.p[h] = f2_add_rn(gx.p[h], f2_mul_alone(f2_pack(c.a, c.a), gz.p[h], nz));
+    gx = f2_add_rn(gx, f2_mul_alone(f2_pack(c.a, c.a), gz, nz));
   } else if (c.op == ADHA_OP_TANH) {
-    LaneVec<M> t;
-    t.load(s + c.vx);
-    const unsigned long long one = f2_pack(1.0f, 1.0f);
-#pragma unroll
-    for (int h = 0; h < H; ++h)
-      gx.p[h] = f2_add_rn(gx.p[h], f2_mul_alone(gz.p[h], f2_sub_rn(one, f2_mul_alone(t.p[h], t.p[h], nz)), nz));
+    const unsigned long long t = lane_load<M>(s + c.vx), one = f2_pack(1.0f, 1.0f);
+    gx = f2_add_rn(gx, f2_mul_alone(gz, f2_sub_rn(one, f2_mul_alone(t, t, nz)), nz));
   } else {
-    LaneVec<M> x, y, gy;
-    x.load(s + c.vx);
-    y.load(s + c.vy);
-#pragma unroll
-    for (int h = 0; h < H; ++h) gx.p[h] = f2_add_rn(gx.p[h], f2_mul_alone(gz.p[h], y.p[h], nz));
-    gx.store(g + c.gx);
-    gy.load(g + c.gy_in);   // after the store: x and y may be the same field
-#pragma unroll
-    for (int h = 0; h < H; ++h) gy.p[h] = f2_add_rn(gy.p[h], f2_mul_alone(gz.p[h], x.p[h], nz));
-    gy.store(g + c.gy);
+    const unsigned long long x = lane_load<M>(s + c.vx), y = lane_load<M>(s + c.vy);
+    lane_store<M>(g + c.gx, f2_add_rn(gx, f2_mul_alone(gz, y, nz)));
+    // after the store: x and y may be the same field
+    lane_store<M>(g + c.gy, f2_add_rn(lane_load<M>(g + c.gy_in), f2_mul_alone(gz, x, nz)));
     return;
   }
-  gx.store(g + c.gx);
+  lane_store<M>(g + c.gx, gx);
 }
 
 // Which of a row's addresses a load or store uses.
@@ -322,10 +297,7 @@ __global__ void __launch_bounds__(kChainThreads) chain_backward_kernel(const __g
   uint8_t* S = smem + chain_tables(a);
   uint8_t* G = S + (a.n_rows + a.n_extra) * R4;
   const int at = lane * M * 4;
-  LaneVec<M> zero;
-#pragma unroll
-  for (int h = 0; h < LaneVec<M>::H; ++h) zero.p[h] = 0ull;
-  zero.store(G + a.n_rows * R4 + at);   // the row of zeros
+  lane_store<M>(G + a.n_rows * R4 + at, 0ull);   // the row of zeros
   for (int64_t c = blockIdx.x; c < a.n_chunks; c += gridDim.x) {
     const int64_t i0 = c * R;
     const bool whole = i0 + R <= a.n;
@@ -366,7 +338,7 @@ __global__ void __launch_bounds__(kChainThreads) chain_backward_kernel(const __g
       nadj = adj[s + 1];
       chain_adjoint<M>(c, S + at, G + at, a.neg_zero);
     }
-    for (uint64_t left = a.zero_rows; left; left &= left - 1) zero.store(G + (__ffsll((long long)left) - 1) * R4 + at);
+    for (uint64_t left = a.zero_rows; left; left &= left - 1) lane_store<M>(G + (__ffsll((long long)left) - 1) * R4 + at, 0ull);
     __syncwarp();
     if (whole) {
       store_spans<M>(gout, a.n_span[3], G, i0, lane);

@@ -196,7 +196,7 @@ struct ChainSpan {       // an array of 4-byte values that one row of a chunk co
 };
 struct ChainArgs {
   int64_t n, n_chunks;   // records; chunks counting the ragged one
-  int64_t pitch;         // floats per row of `saved`: n rounded up to whole 128-record chunks
+  int64_t pitch;         // floats per row of `saved`: n rounded up to a multiple of 128 (whole chunks, aligned rows)
   float* saved;
   unsigned long long neg_zero;   // the pair (-0, -0) (see f2_mul_alone)
   int32_t n_rows, n_sec, n_live, n_extra, n_wide, n_copy;   // n_sec: sections of `sec` or `adj`; n_extra: slots beyond the rows
