@@ -452,11 +452,14 @@ size_t adha_measure_workspace_bytes_for(const adha_schema* schema, int64_t n, co
  * the fastest enters the table and the library's tuning cache, which later
  * launches of the same section (or pair of layouts), layout and size class use.
  * With ADHA_MEASURE_DIFFERENTIABLE (fp32 schemas whose sections are all axpb,
- * mul or tanh) the table prices a forward + backward step instead: a section
- * costs its forward launch with the overwritten values saved plus its adjoint
- * kernel (adha_section_backward) in that layout, and a remap edge costs the
- * remap plus its inverse (the gradients travel back through it), so
- * remap_ns[a][b] = remap_ns[b][a]; fused runs are not timed then.
+ * mul or tanh) the table prices a forward + backward step, section by section,
+ * instead: a section costs its forward launch with the overwritten values saved
+ * plus its adjoint kernel (adha_section_backward) in that layout, and a remap
+ * edge costs the remap plus its inverse (the gradients travel back through it),
+ * so remap_ns[a][b] = remap_ns[b][a]; fused runs are not timed then.  Consecutive
+ * sections run as one chain run (adha_chain_forward) cost less than these sums,
+ * and hardly more for more sections: for long chains the sums overstate the
+ * sections against the remaps, and uniform plans are worth timing beside PDL's.
  * Synchronizes `stream`; *out is a library-owned table (adha_free).
  */
 int adha_measure(const adha_schema* schema, int64_t n, const adha_layout* in_layout, void* const* in_ptrs,
@@ -757,7 +760,9 @@ int adha_tune_clear(void);
  * keys start with S, remap keys with M and carry records per chunk (0: by size;
  * 1024: the library's own choice of kernel) and the piece-table bits as mode) into buf
  * (len bytes, NUL-terminated); *needed = bytes required.  buf may be NULL to
- * ask for the size.  Host only. */
+ * ask for the size.  A remap entry other than 1024 holds its pair of layouts to
+ * the schedule kernel, also one written by a version that had no other: clear
+ * the cache and measure again to have both compared.  Host only. */
 int adha_tune_export(char* buf, size_t len, size_t* needed);
 
 /* Adds the entries of a text made by adha_tune_export to the cache.  Host only. */
