@@ -920,7 +920,8 @@ static int check_section(const Layout& L, const adha_section* s, int64_t n, bool
 // * 64: mix 372 -> 150, drift (6 accesses) 93 -> 75, kick (4) 82 -> 76, bin (3) 71 -> 74, axpb 68 -> 74;
 // * 32: mix 114 -> 79, drift (9) 63 -> 55, gather (6) 87 -> 83, ke (4) 31 -> 39, bin (3) 27 -> 36, tanh 38 -> 48;
 //   96: mix of 24 fields 329 -> 235, reading 24 and writing one 134 -> 124, axpb 99 -> 109; fp64 fields conflict
-//   half as often (32 bytes, mix of 4: 82 -> 91);
+//   half as often (32 bytes, mix of 4, two CTAs per SM instead of three: 82 -> 91; in 80-byte records, four instead
+//   of five: 180 -> 168);
 // * assign reads four features at a time where they lie together (32 bytes 43 -> 46, 64: 87 -> 71, 96: 98 ->
 //   102; 32 bytes in another order 75 -> 70), and in reduce the lanes read one record's consecutive words, only the
 //   membership a column (four 32-byte structs 109 -> 114, 128: 109 -> 105).
@@ -929,9 +930,8 @@ static bool section_room(const Layout& L, int g, const adha_section* s, uint64_t
   if (!staged_room(stride)) return false;
   if (stride % 128 == 0) return true;
   if (s->op == ADHA_OP_REDUCE) return false;
-  int halves = 0;   // accesses per record, two for each, one for an fp64 field at 32, 96, ... bytes
-  for (int f : L.groups[g])
-    halves += (has(staged, f) + (writeback && has(s->write_mask, f))) * (stride % 64 && dtype_size(L.dtype[f]) == 8 ? 1 : 2);
+  int accesses = 0;   // per record
+  for (int f : L.groups[g]) accesses += has(staged, f) + (writeback && has(s->write_mask, f));
   if (s->op == ADHA_OP_ASSIGN) {
     std::vector<int> x;   // the features in order
     for (int f = 0; f < L.F; ++f)
@@ -939,10 +939,10 @@ static bool section_room(const Layout& L, int g, const adha_section* s, uint64_t
     for (size_t j = 0; j + 4 <= x.size(); j += 4) {
       bool four = L.group_of[x[j]] == g && L.offset_of[x[j]] % 16 == 0;
       for (int b = 1; b < 4 && four; ++b) four = L.group_of[x[j + b]] == g && L.offset_of[x[j + b]] == L.offset_of[x[j]] + 4 * b;
-      if (four) halves -= 6;
+      if (four) accesses -= 3;
     }
   }
-  return stride % 64 == 0 ? halves >= 8 : 8 * halves >= 3 * stride;
+  return stride % 64 == 0 ? accesses >= 4 : 16 * accesses >= 3 * stride;
 }
 
 int check_section_layout(const Layout& L, const adha_section* s, int64_t n) { return check_section(L, s, n, false); }
@@ -1048,7 +1048,7 @@ static int plan_section(const Layout& L, void* const* ptrs, const adha_section* 
       a.f[f].wsm = 0;
       a.f[f].dtype = L.dtype[f];
     }
-    int off = 0, odd_rooms = 0;
+    int off = 0, odd_rooms = 0, least = 2;   // least: CTAs per SM that the room must leave
     a.n_writeback = 0;
     for (int k = 0; k < a.n_load; ++k) {
       const int g = groups[k];
@@ -1066,6 +1066,7 @@ static int plan_section(const Layout& L, void* const* ptrs, const adha_section* 
       const bool odd = L.stride[g] % 64 != 0;
       a.pad[k] = room > (odd ? 1 : 0) && section_room(L, g, s, staged, a.writeback[k]) ? 1 : 0;
       if (odd) odd_rooms += a.pad[k];
+      if (odd && a.pad[k] && L.dtype[L.groups[g][0]] == ADHA_F64) least = 3;
       const int stride = L.stride[g] + 16 * a.pad[k];
       for (int f : L.groups[g]) {
         a.f[f].s0 = off + L.offset_of[f];
@@ -1094,8 +1095,8 @@ static int plan_section(const Layout& L, void* const* ptrs, const adha_section* 
       if ((has(staged, f) || has(s->write_mask, f)) && L.groups[L.group_of[f]].size() != 1) a.vec = 0;
     plan->smem = section_smem_bytes(a);
     // not where it leaves an SM with one CTA instead of two (two 96-byte structs 663 -> 915 us)
-    const size_t odd_bytes = (size_t)kWarps * buffers * R * 16 * odd_rooms, two = kSmemPerSM / 2 - kSmemReservedPerCTA;
-    if (odd_rooms && plan->smem > two && plan->smem - odd_bytes <= two) {
+    const size_t odd_bytes = (size_t)kWarps * buffers * R * 16 * odd_rooms, most = kSmemPerSM / least - kSmemReservedPerCTA;
+    if (odd_rooms && plan->smem > most && plan->smem - odd_bytes <= most) {
       room = 1;
       continue;
     }

@@ -2,8 +2,9 @@
 // Table 4: CPU-ODS(1-3) remap GPU-ODS(4-7)).
 //
 // Two kernels: column_kernel, lane = record, the default (described below), and remap_kernel, by an
-// element schedule, for tuned or forced shapes and records too wide for the other.  In both every warp
-// works alone on chunks of R consecutive records, so that the main loop has no block-wide barrier.
+// element schedule, for tuned or forced shapes, records too wide for the other and the pairs of layouts
+// that it moves faster (schedule_faster in capi.cu).  In both every warp works alone on chunks of R
+// consecutive records, so that the main loop has no block-wide barrier.
 // remap_kernel (R a multiple of 8):
 //   1. the warp copies the chunk's slice of every source group into its own shared buffer with
 //      16-byte cp.async (coalesced: lane l moves bytes 16l, 16l+512, ...): one chunk ahead of
