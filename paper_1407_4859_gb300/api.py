@@ -85,13 +85,16 @@ def _ptrs(bufs):
     return (ctypes.c_void_p * max(1, len(bufs)))(*_addresses(bufs))
 
 
+# The current stream's handle without a Stream object around it (2 us of a launch), where this torch has the
+# calls: they are no public ones.
+_RAW_STREAM = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_RAW_DEVICE = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream_ptr(stream):
     if stream is None:
-        # the current stream's handle without a Stream object around it (2 us of a launch), where this torch has
-        # the call: it is no public one
-        raw, device = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
-        if raw and device and torch.cuda.is_initialized():
-            return ctypes.c_void_p(raw(device()))
+        if _RAW_STREAM and _RAW_DEVICE and torch.cuda.is_initialized():
+            return ctypes.c_void_p(_RAW_STREAM(_RAW_DEVICE()))
         stream = torch.cuda.current_stream()
     return ctypes.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
 
